@@ -225,6 +225,16 @@ int sqg_search_ex(const sqg_index *ix, const float *queries, int nq, const int32
                   uint32_t *out_ids, float *out_dists, const sqg_search_params *params, void *workspace,
                   size_t ws_bytes, sqg_query_stats *stats, sqg_stream_t stream);
 
+/* sqg_search_ex for a batch with one k and one ef: the values come by
+ * argument instead of as device arrays, so nothing has to be filled or copied
+ * before the call.  The same results as sqg_search_ex with k[i] = k, ef[i] =
+ * ef and params->uniform_k = k (params->uniform_k must be 0 or k; a max_ef of
+ * 0 means ef); with a workspace the call is asynchronous and allocates
+ * nothing.  1 <= k <= SQG_MAX_K, ef >= 1. */
+int sqg_search_uniform(const sqg_index *ix, const float *queries, int nq, int k, int ef, uint32_t *out_ids,
+                       float *out_dists, const sqg_search_params *params, void *workspace, size_t ws_bytes,
+                       sqg_query_stats *stats, sqg_stream_t stream);
+
 /* Device workspace bytes sqg_search_ex needs for nq queries with the given
  * bounds and these parameters (NULL = defaults; their max_k/max_ef fields are
  * ignored).  The tuning fields (warps_per_block, visited_smem_log2, lean) set

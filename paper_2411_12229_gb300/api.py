@@ -21,7 +21,21 @@ def _stream_ptr(stream) -> int:
     return int(s.cuda_stream)
 
 
-def _i32(x, nq: int, device) -> torch.Tensor:
+def _scalar(x) -> int | None:
+    """x as an int32 value if it is one number, else None."""
+    if isinstance(x, torch.Tensor) or np.ndim(x) != 0:
+        return None
+    return int(np.asarray(x, dtype=np.int32))
+
+
+def _i32(x, nq: int, device, stream=None) -> torch.Tensor:
+    """nq int32 values on the device: a tensor or array of them, or one number
+    for all (filled on the stream that will read it: a host copy of the array
+    would wait for everything the stream still has to do)."""
+    one = _scalar(x)
+    if one is not None:
+        with torch.cuda.stream(stream):
+            return torch.full((nq,), one, dtype=torch.int32, device=device)
     if isinstance(x, torch.Tensor):
         t = x.to(device=device, dtype=torch.int32).contiguous()
     else:
@@ -116,9 +130,21 @@ class Index:
             raise ValueError(f"queries must be a CUDA float32 tensor of shape (nq, {self.d})")
         queries = queries.contiguous()
         nq, dev = queries.shape[0], queries.device
-        kt, et = _i32(k, nq, dev), _i32(ef, nq, dev)
-        uniform = not isinstance(k, torch.Tensor) and np.ndim(k) == 0
+        k1, ef1 = _scalar(k), _scalar(ef)
+        uniform = k1 is not None
         uk = int(kw.get("uniform_k", 0))  # rows of uk slots whatever k[] holds
+        p = self.params(**kw)
+        if uniform and p.max_k == 0:
+            p.max_k = int(k)
+        if uniform and "uniform_k" not in kw and p.max_k == int(k):
+            p.uniform_k = int(k)  # one k for the batch: outputs at i * k, no planning kernel
+        if ef1 is not None and p.max_ef == 0:
+            p.max_ef = int(ef)
+        # one k and one ef: passed by value, no arrays (ef < 1 or another
+        # uniform_k keeps the arrays and the checks made on them)
+        by_value = uniform and ef1 is not None and ef1 >= 1 and 1 <= k1 <= B.MAX_K and p.uniform_k == k1
+        if not by_value:
+            kt, et = _i32(k, nq, dev, stream), _i32(ef, nq, dev, stream)
         if out is None:  # (with `out` given nothing here waits on the device)
             total = uk * nq if uk else int(k) * nq if uniform else int(kt.clamp(0, B.MAX_K).sum().item())
             ids = torch.empty(total, dtype=torch.int32, device=dev)
@@ -126,18 +152,17 @@ class Index:
         else:
             ids, dists = out
         st = torch.empty((nq, 2), dtype=torch.int32, device=dev) if stats else None
-        p = self.params(**kw)
-        if uniform and p.max_k == 0:
-            p.max_k = int(k)
-        if uniform and "uniform_k" not in kw and p.max_k == int(k):
-            p.uniform_k = int(k)  # one k for the batch: outputs at i * k, no planning kernel
-        if not isinstance(ef, torch.Tensor) and np.ndim(ef) == 0 and p.max_ef == 0:
-            p.max_ef = int(ef)
         ws_ptr, ws_bytes = (workspace.data_ptr(), workspace.numel() * workspace.element_size()) \
             if workspace is not None else (None, 0)
-        rc = B.lib().sqg_search_ex(self._h, queries.data_ptr(), nq, kt.data_ptr(), et.data_ptr(), ids.data_ptr(),
-                                   dists.data_ptr(), C.byref(p), ws_ptr, ws_bytes,
-                                   st.data_ptr() if st is not None else None, _stream_ptr(stream))
+        st_ptr = st.data_ptr() if st is not None else None
+        if by_value:
+            rc = B.lib().sqg_search_uniform(self._h, queries.data_ptr(), nq, k1, ef1, ids.data_ptr(),
+                                            dists.data_ptr(), C.byref(p), ws_ptr, ws_bytes, st_ptr,
+                                            _stream_ptr(stream))
+        else:
+            rc = B.lib().sqg_search_ex(self._h, queries.data_ptr(), nq, kt.data_ptr(), et.data_ptr(),
+                                       ids.data_ptr(), dists.data_ptr(), C.byref(p), ws_ptr, ws_bytes, st_ptr,
+                                       _stream_ptr(stream))
         B.check(rc, "sqg_search_ex")
         if uniform or uk:
             ids, dists = ids.view(nq, uk or int(k)), dists.view(nq, uk or int(k))
@@ -158,7 +183,7 @@ class Index:
         and, with path_cap > 0, path (nq, path_cap; -1 past the last hop)."""
         queries = self.fit_queries(queries)
         nq, dev = queries.shape[0], queries.device
-        kt, et = _i32(k, nq, dev), _i32(ef, nq, dev)
+        kt, et = _i32(k, nq, dev, stream), _i32(ef, nq, dev, stream)
         ids = torch.empty(nq * k, dtype=torch.int32, device=dev)
         dists = torch.empty(nq * k, dtype=torch.float32, device=dev)
         st = torch.empty((nq, 2), dtype=torch.int32, device=dev)
@@ -168,7 +193,7 @@ class Index:
             hits = torch.full((nq, trace_cap), -1, dtype=torch.int32, device=dev)
             cnt = torch.zeros(nq, dtype=torch.int32, device=dev)
         path = torch.full((nq, path_cap), -1, dtype=torch.int32, device=dev) if path_cap > 0 else None
-        p = self.params(max_k=k, max_ef=ef, **kw)
+        p = self.params(max_k=k, max_ef=ef, **{"uniform_k": k, **kw})  # rows of k: no planning kernel
         gtp, gtk = (gt.data_ptr(), gt.shape[1]) if gt is not None else (None, 0)
         ptr = lambda t: t.data_ptr() if t is not None else None  # noqa: E731
         rc = B.lib().sqg_search_trace(self._h, queries.contiguous().data_ptr(), nq, kt.data_ptr(), et.data_ptr(),

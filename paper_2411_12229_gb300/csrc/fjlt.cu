@@ -20,8 +20,10 @@ constexpr int kWarps = 4;
 
 template <int E>  // d = 32 E
 __global__ void __launch_bounds__(kWarps * 32)
-    fjlt_kernel(const float *__restrict__ q, const float *__restrict__ signs, float *__restrict__ out, int nq) {
+    fjlt_kernel(const float *__restrict__ q, const float *__restrict__ signs, float *__restrict__ out, int nq,
+                unsigned int *queue) {
     constexpr int d = 32 * E;
+    if (queue && blockIdx.x == 0 && threadIdx.x == 0) *queue = 0u;  // the search's work queue
     const int lane = threadIdx.x & 31;
     const int qi = blockIdx.x * kWarps + (threadIdx.x >> 5);
     if (qi >= nq) return;
@@ -61,8 +63,8 @@ __global__ void __launch_bounds__(kWarps * 32)
 }
 
 template <int E>
-cudaError_t launch_e(const float *q, const float *signs, float *out, int nq, cudaStream_t s) {
-    fjlt_kernel<E><<<(nq + kWarps - 1) / kWarps, kWarps * 32, 0, s>>>(q, signs, out, nq);
+cudaError_t launch_e(const float *q, const float *signs, float *out, int nq, unsigned int *queue, cudaStream_t s) {
+    fjlt_kernel<E><<<(nq + kWarps - 1) / kWarps, kWarps * 32, 0, s>>>(q, signs, out, nq, queue);
     return cudaGetLastError();
 }
 
@@ -71,16 +73,17 @@ cudaError_t launch_e(const float *q, const float *signs, float *out, int nq, cud
 namespace sqg {
 
 // q' for nq queries (nq x d, row-major) into out; d a power of 2 in 32..2048.
-cudaError_t launch_fjlt(const float *q, const float *signs, float *out, int nq, int d, cudaStream_t s) {
+cudaError_t launch_fjlt(const float *q, const float *signs, float *out, int nq, int d, unsigned int *queue,
+                        cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
     switch (d) {
-        case 32: return launch_e<1>(q, signs, out, nq, s);
-        case 64: return launch_e<2>(q, signs, out, nq, s);
-        case 128: return launch_e<4>(q, signs, out, nq, s);
-        case 256: return launch_e<8>(q, signs, out, nq, s);
-        case 512: return launch_e<16>(q, signs, out, nq, s);
-        case 1024: return launch_e<32>(q, signs, out, nq, s);
-        case 2048: return launch_e<64>(q, signs, out, nq, s);
+        case 32: return launch_e<1>(q, signs, out, nq, queue, s);
+        case 64: return launch_e<2>(q, signs, out, nq, queue, s);
+        case 128: return launch_e<4>(q, signs, out, nq, queue, s);
+        case 256: return launch_e<8>(q, signs, out, nq, queue, s);
+        case 512: return launch_e<16>(q, signs, out, nq, queue, s);
+        case 1024: return launch_e<32>(q, signs, out, nq, queue, s);
+        case 2048: return launch_e<64>(q, signs, out, nq, queue, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -406,8 +406,9 @@ constexpr int kMaxWords = kMaxD / 32;
 __global__ void __launch_bounds__(kQxWarps * 32)
     quantize_exact_kernel(const float *__restrict__ q, const float *__restrict__ rot, const float *__restrict__ qa,
                           int nq, int d, float err_scale, uint32_t *__restrict__ planes, float4 *__restrict__ scal,
-                          uint32_t *__restrict__ recomputed, int plane_major) {
+                          uint32_t *__restrict__ recomputed, int plane_major, unsigned int *queue) {
     extern __shared__ __align__(16) unsigned char qxsm[];
+    if (queue && blockIdx.x == 0 && threadIdx.x == 0) *queue = 0u;  // the search's work queue
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int qi = blockIdx.x * kQxWarps + wib;
     if (qi >= nq) return;
@@ -589,14 +590,15 @@ cudaError_t launch_rotate_tc(const float *q, const float *rot_hi, const float *r
 }
 
 cudaError_t launch_quantize_exact(const float *q, const float *rot, const float *qa, int nq, int d, uint32_t *planes,
-                                  float4 *scal, uint32_t *recomputed, bool plane_major, cudaStream_t s) {
+                                  float4 *scal, uint32_t *recomputed, bool plane_major, unsigned int *queue,
+                                  cudaStream_t s) {
     if (d > kMaxD || d % 32 != 0) return cudaErrorInvalidValue;
     if (nq <= 0) return cudaSuccess;
     const size_t smem = kQxWarps * QxLayout(d).warp;
     cudaError_t e = cudaFuncSetAttribute(quantize_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     quantize_exact_kernel<<<(nq + kQxWarps - 1) / kQxWarps, kQxWarps * 32, smem, s>>>(
-        q, rot, qa, nq, d, rotate_tc_err_scale(d), planes, scal, recomputed, plane_major ? 1 : 0);
+        q, rot, qa, nq, d, rotate_tc_err_scale(d), planes, scal, recomputed, plane_major ? 1 : 0, queue);
     return cudaGetLastError();
 }
 

@@ -46,7 +46,7 @@ struct SearchArgs {
     const float *queries;  // nq x d
     const float *qrot;     // nq x d, P^-1 q
     int nq;
-    const int32_t *k, *ef;
+    const int32_t *k, *ef;     // nq each, or both null: every query has k = uniform_k and ef = one_ef
     const long long *offsets;  // nq: output offset of each query
     uint32_t *out_ids;
     float *out_dists;
@@ -55,6 +55,7 @@ struct SearchArgs {
     unsigned int *queue_head;
     int max_k, max_ef, hop_cap;
     int uniform_k;        // > 0: every k[i] equals it, outputs at i * uniform_k (offsets unused)
+    int one_ef;           // the batch's one ef where k and ef are null
     uint32_t hash_bits;   // full visited table: 2^hash_bits >= 2 * hop cap + 1
     uint32_t shash_bits;  // shared-memory table (<= hash_bits)
     uint32_t *ghash;      // per-warp full tables in global memory when shash_bits < hash_bits
@@ -547,7 +548,7 @@ __global__ void __launch_bounds__(128, (LEAN ? 8 : (CH <= 2 ? 5 : 3))) search_ke
         qi = tm.shfl(qi, 0);
         if (qi >= a.nq) break;
 
-        const int k = a.k[qi], ef = a.ef[qi];
+        const int k = a.k ? a.k[qi] : a.uniform_k, ef = a.ef ? a.ef[qi] : a.one_ef;
         const long long off = a.uniform_k ? (long long)qi * a.uniform_k : a.offsets[qi];
         uint32_t status = 0;
         if (!(k >= 1 && k <= a.max_k && ef >= k && ef <= a.max_ef && (!a.uniform_k || k == a.uniform_k))) {
@@ -1011,11 +1012,14 @@ __global__ void __launch_bounds__(128, (LEAN ? 8 : (CH <= 2 ? 5 : 3))) search_ke
 float rotate_tc_err_scale(int d);
 cudaError_t launch_split_tf32(const float *x, float *hi, float *lo, size_t n, cudaStream_t s);
 // The fast JLT on the query side (fjlt.cu); d a power of 2 in 32..2048.
-cudaError_t launch_fjlt(const float *q, const float *signs, float *out, int nq, int d, cudaStream_t s);
+// The last kernel before the search also sets its work-queue head (`queue`, or null) to 0: one launch fewer.
+cudaError_t launch_fjlt(const float *q, const float *signs, float *out, int nq, int d, unsigned int *queue,
+                        cudaStream_t s);
 cudaError_t launch_rotate_tc(const float *q, const float *rot_hi, const float *rot_lo, float *out, int nq, int d,
                              uint32_t *status, cudaStream_t s);
 cudaError_t launch_quantize_exact(const float *q, const float *rot, const float *qa, int nq, int d, uint32_t *planes,
-                                  float4 *scal, uint32_t *recomputed, bool plane_major, cudaStream_t s);
+                                  float4 *scal, uint32_t *recomputed, bool plane_major, unsigned int *queue,
+                                  cudaStream_t s);
 cudaError_t launch_search_nb1(int ch, dim3 grid, dim3 block, size_t smem, cudaStream_t s, const SearchArgs &a);
 cudaError_t launch_search_nb2(int ch, dim3 grid, dim3 block, size_t smem, cudaStream_t s, const SearchArgs &a);
 cudaError_t search_occupancy_nb1(int ch, int block, size_t smem, int *blocks_per_sm);

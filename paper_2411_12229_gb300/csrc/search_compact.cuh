@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
         if (lane == 0) qi = (int)atomicAdd(a.queue_head, 1u);
         qi = __shfl_sync(kFull, qi, 0);
         if (qi >= a.nq) break;
-        const int k = a.k[qi], ef = a.ef[qi];
+        const int k = a.k ? a.k[qi] : a.uniform_k, ef = a.ef ? a.ef[qi] : a.one_ef;
         const long long off = a.uniform_k ? (long long)qi * a.uniform_k : a.offsets[qi];
         uint32_t status = 0;
         if (!(k >= 1 && k <= a.max_k && ef >= k && ef <= a.max_ef && (!a.uniform_k || k == a.uniform_k))) {

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -32,11 +33,22 @@ struct sqg_index {
     uint32_t *d_status;
     int num_sms;
     size_t smem_optin;
+    // Scratch of calls without a caller's workspace.  The device's default
+    // pool hands its memory back at every synchronization, so each call paid
+    // the driver 110-190 us for a fresh mapping.  This pool, owned by the
+    // handle and destroyed with it, keeps up to kPoolKeep bytes mapped between
+    // calls, which then take 2-3 us to get their scratch; it serves the handle
+    // from its second call on, so that a handle made for one batch (index
+    // construction loads one per iteration) keeps nothing.  Order on streams
+    // and thread safety are the stream-ordered allocator's own.
+    cudaMemPool_t pool;
+    mutable std::atomic<bool> scratch_taken{false};
 };
 
 namespace {
 
 constexpr int kPlanThreads = 1024;
+constexpr uint64_t kPoolKeep = 256ull << 20;  // the 16,384-query candidate search at ef 400 takes 110 MB
 
 struct DeviceGuard {
     int prev = -1;
@@ -52,6 +64,16 @@ struct DeviceGuard {
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // The kernels read query rows as float4 and workspace regions as uint4.
 inline bool aligned(const void *p, size_t a) { return reinterpret_cast<uintptr_t>(p) % a == 0; }
+
+// Stream-ordered scratch (released with cudaFreeAsync).  Under stream capture
+// the memory is the graph's own, from the default pool's properties.
+cudaError_t scratch_alloc(const sqg_index *ix, void **p, size_t bytes, cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (ix->pool && ix->scratch_taken.exchange(true, std::memory_order_relaxed) &&
+        cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone)
+        return cudaMallocFromPoolAsync(p, bytes, ix->pool, s);
+    return cudaMallocAsync(p, bytes, s);
+}
 
 // ---------------------------------------------------------------- kernels
 
@@ -170,7 +192,8 @@ __global__ void mlp_transpose_kernel(const float *__restrict__ src, float *__res
 // no bit.
 constexpr int kRotT = 64, kRotK = 32;
 __global__ void __launch_bounds__(256) rotate_kernel(const float *__restrict__ q, const float *__restrict__ rot,
-                                                     float *__restrict__ out, int nq, int d) {
+                                                     float *__restrict__ out, int nq, int d, unsigned int *queue) {
+    if (queue && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *queue = 0u;  // the search's work queue
     __shared__ __align__(16) float As[2][kRotK][kRotT + 4];  // [buffer][j][row]
     __shared__ __align__(16) float Bs[2][kRotK][kRotT + 4];  // [buffer][j][col]
     const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
@@ -503,12 +526,13 @@ const float *queries_for(const sqg_index *ix, const float *queries, int nq, floa
 }
 
 // q' on the CUDA cores: the fast JLT for a version-2 index, else the dense
-// P^-1 q in the canonical chunked order.
-cudaError_t rotate_simt(const sqg_index *ix, const float *queries, float *out, int nq, cudaStream_t stream) {
+// P^-1 q in the canonical chunked order.  Clears `queue` (or null).
+cudaError_t rotate_simt(const sqg_index *ix, const float *queries, float *out, int nq, unsigned int *queue,
+                        cudaStream_t stream) {
     const int d = (int)ix->lay.d;
-    if (ix->fjlt) return launch_fjlt(queries, ix->d_signs, out, nq, d, stream);
+    if (ix->fjlt) return launch_fjlt(queries, ix->d_signs, out, nq, d, queue, stream);
     dim3 rg((d + kRotT - 1) / kRotT, (nq + kRotT - 1) / kRotT);
-    rotate_kernel<<<rg, 256, 0, stream>>>(queries, ix->d_rot, out, nq, d);
+    rotate_kernel<<<rg, 256, 0, stream>>>(queries, ix->d_rot, out, nq, d, queue);
     return cudaGetLastError();
 }
 
@@ -613,6 +637,20 @@ extern "C" int sqg_index_load(const char *path, int device, sqg_index **out) {
         return SQG_ERR_OOM;
     }
     cudaMemset(ix->d_status, 0, sizeof(uint32_t));
+    {  // a device without its own pools serves the scratch from the default one
+        cudaMemPoolProps props;
+        std::memset(&props, 0, sizeof(props));
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        uint64_t keep = kPoolKeep;
+        if (cudaMemPoolCreate(&ix->pool, &props) != cudaSuccess) {
+            ix->pool = nullptr;
+            cudaGetLastError();
+        } else if (cudaMemPoolSetAttribute(ix->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+        }
+    }
     if (ix->fjlt) {  // the fast JLT's signs, from the rotation seed
         std::vector<float> sg(3 * (size_t)L.d);
         for (uint32_t r = 0; r < 3; ++r)
@@ -690,6 +728,7 @@ extern "C" void sqg_index_free(sqg_index *ix) {
     if (ix->d_rot_lo) cudaFree(ix->d_rot_lo);
     if (ix->d_signs) cudaFree(ix->d_signs);
     if (ix->d_status) cudaFree(ix->d_status);
+    if (ix->pool) cudaMemPoolDestroy(ix->pool);
     delete ix;
 }
 
@@ -743,10 +782,11 @@ static int search_impl(const sqg_index *ix, const float *queries, int nq, const 
                        uint32_t *out_ids, float *out_dists, const sqg_search_params *params, void *workspace,
                        size_t ws_bytes, sqg_query_stats *stats, cudaStream_t stream, float *trace_feat,
                        int32_t *trace_hit, int32_t *trace_n, int trace_cap, const uint32_t *gt, int gt_k,
-                       uint32_t *path = nullptr, int path_cap = 0) {
+                       uint32_t *path = nullptr, int path_cap = 0, int one_ef = 0) {
+    // one_ef > 0: k and ef are null, every query has k = params->uniform_k and ef = one_ef
     if (!ix || nq < 0) return SQG_ERR_INVALID_ARG;
     if (nq == 0) return SQG_OK;
-    if (!queries || !k || !ef || !out_ids || !out_dists) return SQG_ERR_INVALID_ARG;
+    if (!queries || (one_ef == 0 && (!k || !ef)) || !out_ids || !out_dists) return SQG_ERR_INVALID_ARG;
     if (!aligned(queries, 16) || (workspace && !aligned(workspace, 256))) return SQG_ERR_INVALID_ARG;
     sqg_search_params p = params ? *params : default_params();
     if (params && p.stop_every == 0) p.stop_every = 1;
@@ -761,7 +801,7 @@ static int search_impl(const sqg_index *ix, const float *queries, int nq, const 
     }
     if (max_k == 0 || max_ef == 0) {  // read the batch's bounds (one stream sync)
         void *tmp = nullptr;
-        if (cudaMallocAsync(&tmp, 8 * (size_t)nq + 256, stream) != cudaSuccess) return SQG_ERR_OOM;
+        if (scratch_alloc(ix, &tmp, 8 * (size_t)nq + 256, stream) != cudaSuccess) return SQG_ERR_OOM;
         int *maxes = reinterpret_cast<int *>(reinterpret_cast<char *>(tmp) + align_up(8 * (size_t)nq, 256));
         plan_kernel<<<1, kPlanThreads, 0, stream>>>(k, ef, nq, reinterpret_cast<long long *>(tmp), maxes);
         int hm[2] = {0, 0};
@@ -777,7 +817,7 @@ static int search_impl(const sqg_index *ix, const float *queries, int nq, const 
     if (rc != SQG_OK) return rc;
     bool own_ws = false;
     if (!workspace) {
-        if (cudaMallocAsync(&workspace, pl.ws_total, stream) != cudaSuccess) return SQG_ERR_OOM;
+        if (scratch_alloc(ix, &workspace, pl.ws_total, stream) != cudaSuccess) return SQG_ERR_OOM;
         own_ws = true;
     } else if (ws_bytes < pl.ws_total) {
         return SQG_ERR_CAPACITY;
@@ -834,6 +874,7 @@ static int search_impl(const sqg_index *ix, const float *queries, int nq, const 
     a.path = path;
     a.path_cap = path_cap;
     a.uniform_k = p.uniform_k;
+    a.one_ef = one_ef;
 
     if (p.uniform_k == 0)  // ragged outputs: the offsets are the prefix sum of k[]
         plan_kernel<<<1, kPlanThreads, 0, stream>>>(k, ef, nq, const_cast<long long *>(a.offsets),
@@ -846,17 +887,17 @@ static int search_impl(const sqg_index *ix, const float *queries, int nq, const 
         if (e == cudaSuccess)
             e = launch_quantize_exact(queries, ix->d_rot, a.qrot, nq, (int)ix->lay.d,
                                       const_cast<uint32_t *>(a.qplanes), const_cast<float4 *>(a.qscal), nullptr,
-                                      false, stream);
+                                      false, a.queue_head, stream);
         if (e != cudaSuccess) {
             if (own_ws) cudaFreeAsync(workspace, stream);
             return SQG_ERR_CUDA;
         }
-    } else if (rotate_simt(ix, queries, const_cast<float *>(a.qrot), nq, stream) != cudaSuccess) {
+    } else if (rotate_simt(ix, queries, const_cast<float *>(a.qrot), nq, a.queue_head, stream) != cudaSuccess) {
         if (own_ws) cudaFreeAsync(workspace, stream);
         return SQG_ERR_CUDA;
     }
-    e = cudaMemsetAsync(a.queue_head, 0, sizeof(unsigned int), stream);
-    if (e == cudaSuccess && p.timing_events[0])
+    e = cudaSuccess;
+    if (p.timing_events[0])
         e = cudaEventRecord(reinterpret_cast<cudaEvent_t>(p.timing_events[0]), stream);
     if (e == cudaSuccess) {
         e = pl.compact && (pl.cbnb == 8 || pl.crk == 4)
@@ -893,6 +934,20 @@ extern "C" int sqg_search_ex(const sqg_index *ix, const float *queries, int nq, 
                        reinterpret_cast<cudaStream_t>(stream), nullptr, nullptr, nullptr, 0, nullptr, 0);
 }
 
+extern "C" int sqg_search_uniform(const sqg_index *ix, const float *queries, int nq, int k, int ef,
+                                  uint32_t *out_ids, float *out_dists, const sqg_search_params *params,
+                                  void *workspace, size_t ws_bytes, sqg_query_stats *stats, sqg_stream_t stream) {
+    if (k < 1 || k > SQG_MAX_K || ef < 1) return SQG_ERR_INVALID_ARG;
+    sqg_search_params p = params ? *params : default_params();
+    if (p.uniform_k != 0 && p.uniform_k != k) return SQG_ERR_INVALID_ARG;
+    p.uniform_k = k;
+    if (p.max_k == 0) p.max_k = k;
+    if (p.max_ef == 0) p.max_ef = ef;
+    return search_impl(ix, queries, nq, nullptr, nullptr, out_ids, out_dists, &p, workspace, ws_bytes, stats,
+                       reinterpret_cast<cudaStream_t>(stream), nullptr, nullptr, nullptr, 0, nullptr, 0, nullptr, 0,
+                       ef);
+}
+
 extern "C" int sqg_search_trace(const sqg_index *ix, const float *queries, int nq, const int32_t *k,
                                 const int32_t *ef, uint32_t *out_ids, float *out_dists,
                                 const sqg_search_params *params, sqg_query_stats *stats, const uint32_t *gt,
@@ -922,7 +977,7 @@ extern "C" int sqg_prepare_queries(const sqg_index *ix, const float *queries, in
         return SQG_ERR_OOM;
     cudaError_t e;
     queries = queries_for(ix, queries, nq, qn, stream, &e);
-    if (e == cudaSuccess) e = rotate_simt(ix, queries, out_qrot, nq, stream);
+    if (e == cudaSuccess) e = rotate_simt(ix, queries, out_qrot, nq, nullptr, stream);
     if (qn) cudaFreeAsync(qn, stream);
     if (e != cudaSuccess) return SQG_ERR_CUDA;
     const int wpb = 4;
@@ -952,7 +1007,7 @@ extern "C" int sqg_prepare_queries_tc(const sqg_index *ix, const float *queries,
         e = launch_rotate_tc(queries, ix->d_rot_hi, ix->d_rot_lo, out_qrot, nq, d, ix->d_status, stream);
     if (e == cudaSuccess)
         e = launch_quantize_exact(queries, ix->d_rot, out_qrot, nq, d, out_planes,
-                                  reinterpret_cast<float4 *>(out_scal), recomputed, true, stream);
+                                  reinterpret_cast<float4 *>(out_scal), recomputed, true, nullptr, stream);
     if (qn) cudaFreeAsync(qn, stream);
     return e == cudaSuccess ? SQG_OK : SQG_ERR_CUDA;
 }
@@ -972,7 +1027,7 @@ extern "C" int sqg_estimate_block(const sqg_index *ix, const float *queries, int
     if (cudaMallocAsync(&qrot, ix->cosine ? 2 * qbytes : qbytes, stream) != cudaSuccess) return SQG_ERR_OOM;
     cudaError_t qe;
     queries = queries_for(ix, queries, nq, qrot + (size_t)nq * d, stream, &qe);
-    if (qe != cudaSuccess || rotate_simt(ix, queries, qrot, nq, stream) != cudaSuccess) {
+    if (qe != cudaSuccess || rotate_simt(ix, queries, qrot, nq, nullptr, stream) != cudaSuccess) {
         cudaFreeAsync(qrot, stream);
         return SQG_ERR_CUDA;
     }
