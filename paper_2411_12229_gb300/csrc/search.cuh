@@ -1007,6 +1007,9 @@ __global__ void __launch_bounds__(128, (LEAN ? 8 : (CH <= 2 ? 5 : 3))) search_ke
     }
 }
 
+// sqg_workspace_size, with or without the deep-beam kernel's own needs (sqg_api.cu).
+size_t workspace_need(const sqg_index *ix, int nq, int max_k, int max_ef, bool allow_deep);
+
 // Host-side launch helpers, defined in the instantiation units.
 // Tensor-core rotation and the exact quantization after it (rotate_tc.cu).
 float rotate_tc_err_scale(int d);
@@ -1051,5 +1054,14 @@ cudaError_t launch_search_compact_big(int ch, int nr, int bnb, int rk, bool stop
                                       cudaStream_t s, const SearchArgs &a);
 cudaError_t search_occupancy_compact_big(int ch, int nr, int bnb, int rk, bool stop, int block, size_t smem,
                                          int *blocks_per_sm);
+// the deep-beam kernel (search_deep.cuh): d <= 2048, out-degree 32 (nr 1) or
+// 64 (nr 2), any ef, k <= 32 (rk 1) or 128 (rk 4), whole warps, multiple
+// estimates, no stop and no feature trace; d > 512 in search_deep_wide.cu
+cudaError_t launch_search_deep(int ch, int nr, int rk, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                               const SearchArgs &a);
+cudaError_t search_occupancy_deep(int ch, int nr, int rk, int block, size_t smem, int *blocks_per_sm);
+cudaError_t launch_search_deep_wide(int ch, int nr, int rk, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                    const SearchArgs &a);
+cudaError_t search_occupancy_deep_wide(int ch, int nr, int rk, int block, size_t smem, int *blocks_per_sm);
 
 }  // namespace sqg

@@ -34,6 +34,10 @@
 
 #include "../../include/sqg.h"
 
+namespace sqg {
+size_t workspace_need(const sqg_index *ix, int nq, int max_k, int max_ef, bool allow_deep);  // sqg_api.cu
+}
+
 namespace {
 
 constexpr size_t kScratchBytes = (size_t)32 << 20;  // 32 MiB on every GPU that loads the library
@@ -74,7 +78,8 @@ extern "C" int sqg_search_noalloc(const sqg_index *ix, const float *queries, int
         return SQG_ERR_INVALID_ARG;
     sqg_info info;
     if (sqg_index_info(ix, &info) != SQG_OK) return SQG_ERR_INVALID_ARG;
-    const size_t need = sqg_workspace_size(ix, nq, max_k, max_ef);
+    size_t need = sqg_workspace_size(ix, nq, max_k, max_ef);
+    if (need > kScratchBytes) need = sqg::workspace_need(ix, nq, max_k, max_ef, false);
     if (need == 0) return SQG_ERR_INVALID_ARG;
     if (need > kScratchBytes) return SQG_ERR_CAPACITY;  // batch too large for the fixed scratch
     void *scratch = nullptr;

@@ -378,6 +378,7 @@ int pick_ch(uint32_t d) {
 struct LaunchPlan {
     int ch, nb, team, warps, grid;
     bool compact;  // the compact kernel (search_compact.cu)
+    bool deep;     // the deep-beam kernel (search_deep.cu)
     int cbnb;      // its beam slots per lane: 2 (ef <= 64), 4 (ef <= 128) or 8 (ef <= 256, d <= 256)
     int crk;       // its result slots per lane: 1 (k <= 32) or 4 (k <= 128, d <= 256)
     size_t smem;
@@ -388,8 +389,11 @@ struct LaunchPlan {
         ws_total;
 };
 
+// What a search records beside its results.
+enum Trace { kNoTrace, kTracePath, kTraceFeatures };
+
 int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_search_params &p, LaunchPlan &pl,
-              bool traced = false) {
+              Trace traced = kNoTrace, bool allow_deep = true) {
     const uint32_t d = ix->lay.d, R = ix->lay.R, bb = ix->lay.block_bytes;
     pl.ch = pick_ch(d);
     pl.nb = (int)(R / 32);
@@ -402,10 +406,19 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
     pl.compact = p.kernel != 1 && pl.team == 32 && pl.ch <= 8 && max_k <= (small_d ? 128 : 32) &&
                  max_ef <= (small_d ? 256 : 128) && p.multi_estimate && !traced && p.prefetch != 2 && p.lean != 2;
     if (p.kernel == 2 && !pl.compact) return SQG_ERR_UNSUPPORTED;
+    // The deep-beam kernel takes what the compact kernel does not (ef past its
+    // range, d > 1024, a recorded path), up to k 128.  Kernel alone, 10k queries
+    // of d 128, general / deep: ef 400 3.36 / 1.57 ms, ef 800 8.55 / 3.17; d 960
+    // ef 256 8.44 / 6.04; 3k queries of d 1536, k 100: ef 100 1.42 / 1.08, ef 400
+    // 5.08 / 3.12, ef 800 10.7 / 5.15.  Within the compact kernel's range the
+    // two are within 8 % at ef 129-256 and the compact one is faster below (ef
+    // 64: 0.36 / 0.42; d 960 ef 112: 2.55 / 2.72).
+    pl.deep = allow_deep && !pl.compact && p.kernel == 0 && pl.team == 32 && max_k <= 128 && p.multi_estimate && !p.stop_mlp &&
+              traced != kTraceFeatures && p.prefetch != 2 && p.lean != 2;
     pl.cbnb = max_ef <= 64 ? 2 : max_ef <= 128 ? 4 : 8;
     pl.crk = max_k <= 32 ? 1 : 4;
     const bool big = pl.compact && (pl.cbnb == 8 || pl.crk == 4);  // search_compact_big.cu
-    if (pl.compact) {
+    if (pl.compact || pl.deep) {
     } else if (pl.team < 32) {
         // smaller teams: d <= 256, the 96-register build, no fused stop network
         if (pl.ch > 2 || p.stop_mlp) return SQG_ERR_UNSUPPORTED;
@@ -438,6 +451,12 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
         a.o_beam = (uint32_t)o; o += 2 * 32 * (size_t)pl.cbnb * 8;
         a.o_res = (uint32_t)o;
         a.o_spos = (uint32_t)o; o += (size_t)R * 8;
+    } else if (pl.deep) {
+        // two front buffers of 2 R packed entries, the main part (o_res; none
+        // if the front holds every beam of the batch), the step's candidates
+        a.o_beam = (uint32_t)o; o += 2 * 2 * (size_t)R * 8;
+        a.o_res = (uint32_t)o; o += max_ef > (int)(2 * R) ? align_up(8 * (size_t)max_ef, 16) : 0;
+        a.o_spos = (uint32_t)o; o += (size_t)R * 8;
     } else {
         a.o_beam = (uint32_t)o; o = align_up(o + 8 * (size_t)max_ef, 16);
         a.o_res = (uint32_t)o; o = align_up(o + 8 * (size_t)max_k, 16);
@@ -463,6 +482,7 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
                                                   blocks)
              : pl.compact && p.stop_mlp ? search_occupancy_compact_stop(pl.ch, pl.nb, pl.cbnb, w * 32, sm, blocks)
              : pl.compact     ? search_occupancy_compact(pl.ch, pl.nb, pl.cbnb, p.lean, w * 32, sm, blocks)
+             : pl.deep        ? search_occupancy_deep(pl.ch, pl.nb, pl.crk, w * 32, sm, blocks)
              : pl.team < 32 ? search_occupancy_team(pl.ch, pl.nb, pl.team, w * 32, sm, blocks)
              : pl.nb == 1   ? search_occupancy_nb1(pl.ch, w * 32, sm, blocks)
                             : search_occupancy_nb2(pl.ch, w * 32, sm, blocks);
@@ -749,13 +769,13 @@ extern "C" int sqg_index_info(const sqg_index *ix, sqg_info *out) {
     return SQG_OK;
 }
 
-extern "C" size_t sqg_workspace_size(const sqg_index *ix, int nq, int max_k, int max_ef) {
+size_t sqg::workspace_need(const sqg_index *ix, int nq, int max_k, int max_ef, bool allow_deep) {
     if (!ix || nq < 0 || max_k < 1 || max_k > SQG_MAX_K || max_ef < max_k || max_ef > SQG_MAX_EF) return 0;
     DeviceGuard g(ix->device);
     // the larger of the plans without and with the learned stop's weights
     LaunchPlan pl;
     sqg_search_params p = default_params();
-    if (make_plan(ix, nq, max_k, max_ef, p, pl) != SQG_OK) return 0;
+    if (make_plan(ix, nq, max_k, max_ef, p, pl, kNoTrace, allow_deep) != SQG_OK) return 0;
     size_t need = pl.ws_total;
     p.kernel = 1;  // the general kernel (its visited tables follow its own residency)
     if (make_plan(ix, nq, max_k, max_ef, p, pl) == SQG_OK) need = std::max(need, pl.ws_total);
@@ -764,6 +784,10 @@ extern "C" size_t sqg_workspace_size(const sqg_index *ix, int nq, int max_k, int
     p.kernel = 0;  // the compact kernel's build with the stop fused
     if (make_plan(ix, nq, max_k, max_ef, p, pl) == SQG_OK) need = std::max(need, pl.ws_total);
     return need;
+}
+
+extern "C" size_t sqg_workspace_size(const sqg_index *ix, int nq, int max_k, int max_ef) {
+    return workspace_need(ix, nq, max_k, max_ef, true);
 }
 
 extern "C" size_t sqg_workspace_size_ex(const sqg_index *ix, int nq, int max_k, int max_ef,
@@ -813,7 +837,12 @@ static int search_impl(const sqg_index *ix, const float *queries, int nq, const 
         if (max_ef == 0) max_ef = std::max(max_k, hm[1]);
     }
     LaunchPlan pl;
-    int rc = make_plan(ix, nq, max_k, max_ef, p, pl, trace_feat != nullptr || path != nullptr);
+    const Trace traced = trace_feat || trace_n ? kTraceFeatures : path ? kTracePath : kNoTrace;
+    int rc = make_plan(ix, nq, max_k, max_ef, p, pl, traced);
+    // more resident warps need more visited tables: a workspace that holds
+    // the general kernel's still serves
+    if (rc == SQG_OK && pl.deep && workspace && ws_bytes < pl.ws_total)
+        rc = make_plan(ix, nq, max_k, max_ef, p, pl, traced, false);
     if (rc != SQG_OK) return rc;
     bool own_ws = false;
     if (!workspace) {
@@ -908,6 +937,8 @@ static int search_impl(const sqg_index *ix, const float *queries, int nq, const 
                                              stream, a)
             : pl.compact ? launch_search_compact(pl.ch, pl.nb, pl.cbnb, p.lean, dim3(pl.grid), dim3(pl.warps * 32),
                                                  pl.smem, stream, a)
+            : pl.deep    ? launch_search_deep(pl.ch, pl.nb, pl.crk, dim3(pl.grid), dim3(pl.warps * 32), pl.smem,
+                                              stream, a)
             : pl.team < 32 ? launch_search_team(pl.ch, pl.nb, pl.team, dim3(pl.grid), dim3(pl.warps * 32), pl.smem,
                                                 stream, a)
             : pl.nb == 1 ? launch_search_nb1(pl.ch, dim3(pl.grid), dim3(pl.warps * 32), pl.smem, stream, a)
