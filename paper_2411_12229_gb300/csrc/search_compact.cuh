@@ -89,40 +89,139 @@ __device__ __forceinline__ void hash_insert_warp(uint32_t *H, uint32_t bits, uin
     }
 }
 
-// S = sum_i b_i qbar_i (Sec. 3.1.1) of neighbours lane + 32 t (t < NR):
-// AND + popc of their code words against the 4 bit-planes, out-degree R =
-// 32 NR (word w of neighbour j at w * R + j); nw <= 4 * CH words, the
-// plane word loaded once for the NR neighbours.
+// A full adder on bit slices: three words of one weight into a word of that
+// weight (xor3) and the carries, a word of twice the weight (maj3).  In PTX
+// so that each is one LOP3: left to itself the compiler spread the majority
+// over the ANDs feeding it (d 960: 5,560 against 4,600 cycles per expansion).
+__device__ __forceinline__ uint32_t xor3(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0x96;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+}
+__device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
+    uint32_t r;
+    asm("lop3.b32 %0, %1, %2, %3, 0xE8;" : "=r"(r) : "r"(a), "r"(b), "r"(c));
+    return r;
+}
+
+// One expansion's exact-distance partial (exact_partial's arithmetic and
+// order) and S = sum_i b_i qbar_i (Sec. 3.1.1) of neighbours lane + 32 n (n <
+// NR), out-degree R = 32 NR: the sums over words w and planes b of 2^b
+// popc(code word w of the neighbour, at w * R + j, AND word w of plane b),
+// nw <= 4 CH words.
+//
+// A POPC holds its pipe for 8 cycles, an AND or ADD the ALU for 2: counted
+// word by word, S of a long code is bound by the POPC pipe (8 cycles per word
+// and plane; d 960 with out-degree 64: 5,850 of an expansion's 8,470 cycles
+// with 12 warps per SM).  For d > 256 full adders in front halve the POPCs
+// for 2 LOP3 each.  Exact partial, S and butterfly at d 960, out-degree 64,
+// cycles per expansion, word by word / here: 4,160 / 2,780 for a lone warp,
+// 6,250 / 4,600 with 12 warps per SM.  A second adder level gains nothing
+// (4,800: the ALU is then the limit).  For d <= 256, where other ALU work
+// dominates a full SM, adders cost more than they save (10k queries of d 128,
+// ef 40: 262 us word by word, 273 with adders).
 template <int CH, int NR>
-__device__ __forceinline__ void estimate_SN(const unsigned char *codes_b, const uint32_t *planes, uint32_t nw,
-                                            int lane, int (&S)[NR]) {
+__device__ __forceinline__ void exact_and_S(const float4 (&qv)[CH], const unsigned char *blk, uint32_t off_codes,
+                                            const uint32_t *planes, uint32_t nch, uint32_t nw, int lane,
+                                            float (&acc)[1], int (&S)[NR]) {
     constexpr uint32_t R = 32 * NR;
-    const uint32_t *codes = reinterpret_cast<const uint32_t *>(codes_b) + lane;
+    const uint32_t *codes = reinterpret_cast<const uint32_t *>(blk + off_codes) + lane;
     const uint4 *pl = reinterpret_cast<const uint4 *>(planes);
-    int s0[NR], s1[NR], s2[NR], s3[NR];
-#pragma unroll
-    for (int t = 0; t < NR; ++t) s0[t] = s1[t] = s2[t] = s3[t] = 0;
-    auto word = [&](uint32_t w) {
-        const uint4 p = pl[w];
-#pragma unroll
-        for (int t = 0; t < NR; ++t) {
-            const uint32_t c = codes[w * R + 32 * t];
-            s0[t] += __popc(c & p.x);
-            s1[t] += __popc(c & p.y);
-            s2[t] += __popc(c & p.z);
-            s3[t] += __popc(c & p.w);
-        }
-    };
     if constexpr (CH <= 2) {
+        exact_partial<CH, 32>(reinterpret_cast<const float4(&)[1][CH]>(qv), reinterpret_cast<const float *>(blk), nch,
+                              Team<32>(lane), acc);
+        int s0[NR], s1[NR], s2[NR], s3[NR];
+#pragma unroll
+        for (int n = 0; n < NR; ++n) s0[n] = s1[n] = s2[n] = s3[n] = 0;
 #pragma unroll
         for (uint32_t w = 0; w < 4 * CH; ++w)
-            if (w < nw) word(w);
-    } else {
-#pragma unroll 4
-        for (uint32_t w = 0; w < nw; ++w) word(w);
-    }
+            if (w < nw) {
+                const uint4 p = pl[w];
 #pragma unroll
-    for (int t = 0; t < NR; ++t) S[t] = s0[t] + 2 * s1[t] + 4 * s2[t] + 8 * s3[t];
+                for (int n = 0; n < NR; ++n) {
+                    const uint32_t c = codes[w * R + 32 * n];
+                    s0[n] += __popc(c & p.x);
+                    s1[n] += __popc(c & p.y);
+                    s2[n] += __popc(c & p.z);
+                    s3[n] += __popc(c & p.w);
+                }
+            }
+#pragma unroll
+        for (int n = 0; n < NR; ++n) S[n] = s0[n] + 2 * s1[n] + 4 * s2[n] + 8 * s3[n];
+    } else {
+        // chunk t: the lane's t-th float4 of the raw vector and words 4 t .. 4
+        // t + 3; `one` carries each plane's sum of weight 1 from word to word
+        const float4 *r4 = reinterpret_cast<const float4 *>(blk);
+        uint32_t one[NR][4];
+        int two[NR][4];  // counts of weight 2
+#pragma unroll
+        for (int n = 0; n < NR; ++n)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                one[n][b] = 0u;
+                two[n][b] = 0;
+            }
+        float s = 0.0f;
+#pragma unroll
+        for (uint32_t t = 0; t < CH; ++t) {
+            if (4 * t >= nw) break;
+            const uint32_t c = lane + 32 * t;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (c < nch) x = r4[c];
+            if (4 * t + 4 <= nw) {
+                uint32_t p[4][4], cw[NR][4];
+#pragma unroll
+                for (uint32_t w = 0; w < 4; ++w) {
+                    const uint4 v = pl[4 * t + w];
+                    p[0][w] = v.x;
+                    p[1][w] = v.y;
+                    p[2][w] = v.z;
+                    p[3][w] = v.w;
+#pragma unroll
+                    for (int n = 0; n < NR; ++n) cw[n][w] = codes[(4 * t + w) * R + 32 * n];
+                }
+#pragma unroll
+                for (int n = 0; n < NR; ++n)
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        const uint32_t a0 = cw[n][0] & p[b][0], a1 = cw[n][1] & p[b][1];
+                        const uint32_t a2 = cw[n][2] & p[b][2], a3 = cw[n][3] & p[b][3];
+                        const uint32_t o = one[n][b], o1 = xor3(o, a0, a1);
+                        two[n][b] += __popc(maj3(o, a0, a1)) + __popc(maj3(o1, a2, a3));
+                        one[n][b] = xor3(o1, a2, a3);
+                    }
+            } else {
+                for (uint32_t w = 4 * t; w < nw; ++w) {
+                    const uint4 v = pl[w];
+#pragma unroll
+                    for (int n = 0; n < NR; ++n) {
+                        const uint32_t e = codes[w * R + 32 * n];
+                        const uint32_t a[4] = {e & v.x, e & v.y, e & v.z, e & v.w};
+#pragma unroll
+                        for (int b = 0; b < 4; ++b) {
+                            two[n][b] += __popc(one[n][b] & a[b]);
+                            one[n][b] ^= a[b];
+                        }
+                    }
+                }
+            }
+            if (c < nch) {
+                const float dx = __fsub_rn(qv[t].x, x.x), dy = __fsub_rn(qv[t].y, x.y);
+                const float dz = __fsub_rn(qv[t].z, x.z), dw = __fsub_rn(qv[t].w, x.w);
+                s = __fmaf_rn(dx, dx, s);
+                s = __fmaf_rn(dy, dy, s);
+                s = __fmaf_rn(dz, dz, s);
+                s = __fmaf_rn(dw, dw, s);
+            }
+        }
+        acc[0] = s;
+#pragma unroll
+        for (int n = 0; n < NR; ++n) {
+            S[n] = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) S[n] += (__popc(one[n][b]) + 2 * two[n][b]) << b;
+        }
+    }
 }
 
 // The key of neighbour j from its S (the estimator of Sec. 3.1.1 and the
@@ -282,13 +381,11 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
             // ---- line 4: exact distance (implicit re-ranking); the neighbours'
             // integer sums S while the distance's butterfly is in flight
             float dacc[1];
-            exact_partial<CH, 32>(reinterpret_cast<const float4(&)[1][CH]>(qv),
-                                  reinterpret_cast<const float *>(blk), nch, tm, dacc);
             uint32_t cid[NR];
             int S[NR];
 #pragma unroll
             for (int t = 0; t < NR; ++t) cid[t] = reinterpret_cast<const uint32_t *>(blk + a.off_ids)[lane + 32 * t];
-            estimate_SN<CH, NR>(blk + a.off_codes, planes, d / 32, lane, S);
+            exact_and_S<CH, NR>(qv, blk, a.off_codes, planes, nch, d / 32, lane, dacc, S);
             const float dist_c = exact_reduce<32>(dacc, tm);
             if (hops == 1) {  // reading R8: the entry's key is its exact distance
                 if (lane == 0) {

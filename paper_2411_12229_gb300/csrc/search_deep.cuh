@@ -196,13 +196,11 @@ __global__ void __launch_bounds__(128, MINB) search_deep_kernel(const SearchArgs
             // ---- line 4: exact distance (implicit re-ranking); the neighbours'
             // integer sums S while the distance's butterfly is in flight
             float dacc[1];
-            exact_partial<CH, 32>(reinterpret_cast<const float4(&)[1][CH]>(qv),
-                                  reinterpret_cast<const float *>(blk), nch, tm, dacc);
             uint32_t cid[NR];
             int S[NR];
 #pragma unroll
             for (int t = 0; t < NR; ++t) cid[t] = reinterpret_cast<const uint32_t *>(blk + a.off_ids)[lane + 32 * t];
-            estimate_SN<CH, NR>(blk + a.off_codes, planes, d / 32, lane, S);
+            exact_and_S<CH, NR>(qv, blk, a.off_codes, planes, nch, d / 32, lane, dacc, S);
             const float dist_c = exact_reduce<32>(dacc, tm);
             if (hops == 1) {  // reading R8: the entry's key is its exact distance
                 if (lane == 0) {
