@@ -103,7 +103,10 @@ int sqg_graph::build_graph_host(const float *data, uint64_t n, uint32_t d, const
         if (sqg_graph::fill_and_write(data, n, d, R, Rr, seed, u, regular, k2, out_adj)) n_fill++;
     });
     // 5. reachability from the entry point
-    const uint64_t repairs = sqg_graph::repair_reachability(n, cand, L, R, entry, out_adj);
+    const uint64_t repairs = sqg_graph::repair_reachability(n, cand, L, R, entry, out_adj, [&](std::vector<uint8_t> &seen) {
+        seen = sqg_graph::reachable_host(n, R, entry, out_adj);
+        return true;
+    });
     if (out_stats) {
         out_stats[0] = deg_sum.load() * 1000 / n;
         out_stats[1] = n_supp.load();

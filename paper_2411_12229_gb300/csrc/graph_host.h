@@ -240,19 +240,36 @@ inline bool fill_and_write(const float *data, uint64_t n, uint32_t d, uint32_t R
     return filled;
 }
 
+// The vertices the entry point reaches, 1 each (any traversal finds the same).
+inline std::vector<uint8_t> reachable_host(uint64_t n, uint32_t R, uint32_t entry, const uint32_t *adj) {
+    std::vector<uint8_t> seen(n, 0);
+    std::vector<uint32_t> stack{entry};
+    seen[entry] = 1;
+    while (!stack.empty()) {
+        const uint32_t u = stack.back();
+        stack.pop_back();
+        for (uint32_t t = 0; t < R; ++t) {
+            const uint32_t v = adj[(uint64_t)u * R + t];
+            if (v != SQG_NO_ID && !seen[v]) { seen[v] = 1; stack.push_back(v); }
+        }
+    }
+    return seen;
+}
+
 // (5) reachability from the entry point: connect each unreachable vertex
 // from a nearby reachable vertex, replacing that vertex's edge whose target
-// has the most other in-edges.  Returns the number of edges replaced.
-inline uint64_t repair_reachability(uint64_t n, const uint32_t *cand, uint32_t L, uint32_t R, uint32_t entry,
-                                    uint32_t *out_adj) {
-    std::vector<uint32_t> in(n, 0);
-    for (uint64_t i = 0; i < n * R; ++i)
-        if (out_adj[i] != SQG_NO_ID) in[out_adj[i]]++;
+// has the most other in-edges.  `reach(seen)` gives the vertices that
+// out_adj's current rows reach; false ends the repair (a failed device).
+// Returns the number of edges replaced.
+template <class Reach>
+uint64_t repair_reachability(uint64_t n, const uint32_t *cand, uint32_t L, uint32_t R, uint32_t entry,
+                             uint32_t *out_adj, Reach reach) {
+    std::vector<uint32_t> in;  // in-edges of every vertex, counted before the first repair
     uint64_t repairs = 0;
     for (int round = 0; round < 16; ++round) {
-        std::vector<uint8_t> seen(n, 0);
-        std::vector<uint32_t> stack{entry};
-        seen[entry] = 1;
+        std::vector<uint8_t> seen;
+        if (!reach(seen)) break;
+        std::vector<uint32_t> stack;
         auto flood = [&]() {
             while (!stack.empty()) {
                 uint32_t u = stack.back();
@@ -263,10 +280,14 @@ inline uint64_t repair_reachability(uint64_t n, const uint32_t *cand, uint32_t L
                 }
             }
         };
-        flood();
         uint64_t fixed = 0;
         for (uint64_t v = 0; v < n; ++v) {
             if (seen[v]) continue;
+            if (in.empty()) {
+                in.assign(n, 0);
+                for (uint64_t i = 0; i < n * R; ++i)
+                    if (out_adj[i] != SQG_NO_ID) in[out_adj[i]]++;
+            }
             uint32_t r = entry;
             for (uint32_t t = 0; t < L; ++t) {
                 uint32_t c = cand[v * L + t];
