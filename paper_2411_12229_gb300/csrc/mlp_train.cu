@@ -2,14 +2,24 @@
 // paper): a 16 -> 64 -> 64 -> 1 ReLU MLP over search-state features,
 // trained with weighted binary cross-entropy and Adam.
 //
-// One block takes a tile of 128 samples and runs the batch as small dense
-// products in shared memory:
+// A block takes tiles of 64 samples and runs each as small dense products in
+// shared memory:
 //   forward  A1 = X W1^T + b1, H1 = relu(A1), A2 = H1 W2^T + b2,
 //            H2 = relu(A2), z = H2 W3 + b3
 //   backward dz = w (sigmoid(z) - y) / sum(w), D2 = (dz W3^T) .* [A2 > 0],
 //            D1 = (D2 W2) .* [A1 > 0]
 //   grads    W3: H2^T dz, W2: D2^T H1, W1: D1^T X, biases: column sums
-// and adds its partial gradient into the global gradient with atomics.
+// The gradient stays in registers over the block's tiles and is added to the
+// global one with atomics at the end.
+//
+// What bounds it: in fp32 the products are 14,400 multiply-adds per sample
+// (8,192 samples: 3.4 us on all SMs).  Every product gives a thread 4 x 4
+// outputs from two 16-byte shared-memory reads per step of the inner
+// dimension (operands kept both ways round where two products read them
+// along different axes); one output per thread with two 4-byte reads per
+// multiply-add, on 64 blocks of 128 samples, took 73 us; this one takes 17 us
+// (8,192 samples: 128 blocks, one tile each; two warps per scheduler, so the
+// barriers between the products are what is left).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -17,33 +27,67 @@
 
 namespace {
 
-constexpr int kIn = SQG_MLP_IN, kH = SQG_MLP_HIDDEN, kTile = 128, kThreads = 256;
+constexpr int kIn = SQG_MLP_IN, kH = SQG_MLP_HIDDEN, kTile = 64, kThreads = 256;
 constexpr int oW1 = 0, ob1 = kH * kIn, oW2 = ob1 + kH, ob2 = oW2 + kH * kH, oW3 = ob2 + kH, ob3 = oW3 + kH;
+constexpr int kLd = kH + 4;  // row pitch: 16-byte aligned, rows a bank quad apart
 
+// [a][b]: a = row, b = contiguous.  i: input, h: first hidden layer, o: second
+// hidden layer, r: sample.
 struct TileSmem {
-    float W[SQG_MLP_NPARAM];
-    float X[kTile][kIn];
-    float A1[kTile][kH + 1];  // pre-activation, later D1
-    float A2[kTile][kH + 1];  // pre-activation, later D2
-    float H1[kTile][kH + 1];
-    float dz[kTile];
-    float lossp[kThreads / 32];
+    float W1ih[kIn][kLd], W2ho[kH][kLd], W2oh[kH][kLd];
+    float b1[kH], b2[kH], W3[kH];
+    float Xir[kIn][kLd], Xri[kTile][kIn + 4];
+    float H1hr[kH][kLd], H1rh[kTile][kLd];
+    float D2or[kH][kLd], D2ro[kTile][kLd];
+    float D1rh[kTile][kLd];
+    float y[kTile], w[kTile];
 };
 
 __device__ __forceinline__ float softplus(float z) { return z > 0.f ? z + log1pf(expf(-z)) : log1pf(expf(z)); }
 
-// sum of the sample weights (one block)
-__global__ void weight_sum_kernel(const float *w, int n, float *out) {
-    __shared__ float part[kThreads / 32];
+// The sum of the sample weights, and the gradient and the loss cleared for the
+// atomics (one block, one launch before the gradient kernel).
+constexpr int kPrepThreads = 1024;
+__global__ void __launch_bounds__(kPrepThreads) prepare_kernel(const float *__restrict__ w, int n, float *wsum,
+                                                               float *grad, float *loss) {
+    __shared__ float part[kPrepThreads / 32];
+    for (int i = threadIdx.x; i < SQG_MLP_NPARAM; i += kPrepThreads) grad[i] = 0.f;
+    if (threadIdx.x == 0 && loss) *loss = 0.f;
     float s = 0.f;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) s += w[i];
+#pragma unroll 8
+    for (int i = threadIdx.x; i < n; i += kPrepThreads) s += w[i];
     for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int i = 0; i < kThreads / 32; ++i) t += part[i];
-        *out = t;
+    if (threadIdx.x < 32) {
+        float t = part[threadIdx.x];
+        for (int o = 16; o >= 1; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+        if (threadIdx.x == 0) *wsum = t;
+    }
+}
+
+// The 4 x 4 values v to dst_ij[r0 + i][c0 + j] and / or dst_ji[c0 + j][r0 + i].
+__device__ __forceinline__ void put4(float *dst_ij, float *dst_ji, const float (&v)[4][4], int r0, int c0) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        *reinterpret_cast<float4 *>(dst_ij + (r0 + i) * kLd + c0) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+        if (dst_ji)
+            *reinterpret_cast<float4 *>(dst_ji + (c0 + i) * kLd + r0) = make_float4(v[0][i], v[1][i], v[2][i], v[3][i]);
+    }
+}
+
+// acc[i][j] += sum over k of A[k][a0 + i] B[k][b0 + j], k < K.
+template <int K>
+__device__ __forceinline__ void outer4(float (&acc)[4][4], const float *A, int a0, const float *B, int b0) {
+#pragma unroll 8
+    for (int k = 0; k < K; ++k) {
+        const float4 a = *reinterpret_cast<const float4 *>(A + k * kLd + a0);
+        const float4 b = *reinterpret_cast<const float4 *>(B + k * kLd + b0);
+        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
     }
 }
 
@@ -53,109 +97,154 @@ __global__ void __launch_bounds__(kThreads) mlp_grad_kernel(const float *__restr
                                                             float *__restrict__ G, float *__restrict__ loss) {
     extern __shared__ __align__(16) unsigned char raw[];
     TileSmem &s = *reinterpret_cast<TileSmem *>(raw);
-    const int tid = threadIdx.x, base = blockIdx.x * kTile;
-    const int rows = min(kTile, n - base);
-    for (int i = tid; i < SQG_MLP_NPARAM; i += kThreads) s.W[i] = P[i];
-    for (int i = tid; i < kTile * kIn; i += kThreads) {
-        int r = i / kIn, c = i % kIn;
-        s.X[r][c] = r < rows ? X[(size_t)(base + r) * kIn + c] : 0.f;
-    }
-    __syncthreads();
-    const float inv_w = 1.0f / *wsum;
-    // A1 = X W1^T + b1
-    for (int i = tid; i < kTile * kH; i += kThreads) {
-        int r = i / kH, o = i % kH;
-        float a = s.W[ob1 + o];
-        for (int c = 0; c < kIn; ++c) a = fmaf(s.W[oW1 + o * kIn + c], s.X[r][c], a);
-        s.A1[r][o] = a;
-        s.H1[r][o] = a > 0.f ? a : 0.f;
-    }
-    __syncthreads();
-    // A2 = H1 W2^T + b2
-    for (int i = tid; i < kTile * kH; i += kThreads) {
-        int r = i / kH, o = i % kH;
-        float a = s.W[ob2 + o];
-        for (int c = 0; c < kH; ++c) a = fmaf(s.W[oW2 + o * kH + c], s.H1[r][c], a);
-        s.A2[r][o] = a;
-    }
-    __syncthreads();
-    // z, loss, dz: one warp per 16 samples, lanes over the 64 hidden units
-    {
-        const int lane = tid & 31, wp = tid >> 5;
-        float lsum = 0.f;
-        for (int r = wp; r < kTile; r += kThreads / 32) {
-            float a0 = s.A2[r][lane], a1 = s.A2[r][lane + 32];
-            float p = s.W[oW3 + lane] * (a0 > 0.f ? a0 : 0.f) + s.W[oW3 + lane + 32] * (a1 > 0.f ? a1 : 0.f);
-            for (int o = 16; o >= 1; o >>= 1) p += __shfl_xor_sync(0xFFFFFFFFu, p, o);
-            const float z = p + s.W[ob3];
-            float dz = 0.f;
-            if (r < rows) {
-                const float yy = y[base + r], ww = w[base + r] * inv_w;
-                lsum += ww * (softplus(z) - yy * z);
-                dz = ww * (1.0f / (1.0f + expf(-z)) - yy);
-            }
-            if (lane == 0) s.dz[r] = dz;
-        }
-        if (lane == 0) s.lossp[wp] = lsum;
-    }
-    __syncthreads();
-    if (tid == 0 && loss) {
-        float t = 0.f;
-        for (int i = 0; i < kThreads / 32; ++i) t += s.lossp[i];
-        atomicAdd(loss, t);
-    }
-    // gW3, gb3 (before A2 is overwritten by D2)
-    if (tid < kH) {
-        float g = 0.f;
-        for (int r = 0; r < kTile; ++r) {
-            float a = s.A2[r][tid];
-            g = fmaf(s.dz[r], a > 0.f ? a : 0.f, g);
-        }
-        atomicAdd(&G[oW3 + tid], g);
-    } else if (tid == kH) {
-        float g = 0.f;
-        for (int r = 0; r < kTile; ++r) g += s.dz[r];
-        atomicAdd(&G[ob3], g);
-    }
-    __syncthreads();
-    // D2 = dz W3 .* [A2 > 0]   (in place of A2)
-    for (int i = tid; i < kTile * kH; i += kThreads) {
-        int r = i / kH, o = i % kH;
-        s.A2[r][o] = s.A2[r][o] > 0.f ? s.dz[r] * s.W[oW3 + o] : 0.f;
-    }
-    __syncthreads();
-    // gW2 = D2^T H1 (64 x 64), gb2 = colsum D2
+    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
+    for (int i = tid; i < kH * kIn; i += kThreads) s.W1ih[i % kIn][i / kIn] = P[oW1 + i];
     for (int i = tid; i < kH * kH; i += kThreads) {
-        int o = i / kH, c = i % kH;
-        float g = 0.f;
-        for (int r = 0; r < kTile; ++r) g = fmaf(s.A2[r][o], s.H1[r][c], g);
-        atomicAdd(&G[oW2 + i], g);
+        const float v = P[oW2 + i];
+        s.W2oh[i / kH][i % kH] = v;
+        s.W2ho[i % kH][i / kH] = v;
     }
     if (tid < kH) {
-        float g = 0.f;
-        for (int r = 0; r < kTile; ++r) g += s.A2[r][tid];
-        atomicAdd(&G[ob2 + tid], g);
+        s.b1[tid] = P[ob1 + tid];
+        s.b2[tid] = P[ob2 + tid];
+        s.W3[tid] = P[oW3 + tid];
     }
-    __syncthreads();  // H1 is read above and overwritten below
-    // D1 = (D2 W2) .* [A1 > 0]   (into H1)
-    for (int i = tid; i < kTile * kH; i += kThreads) {
-        int r = i / kH, c = i % kH;
-        float a = 0.f;
-        for (int o = 0; o < kH; ++o) a = fmaf(s.A2[r][o], s.W[oW2 + o * kH + c], a);
-        s.H1[r][c] = s.A1[r][c] > 0.f ? a : 0.f;  // H1 no longer needed: holds D1
+    const float b3 = P[ob3], inv_w = 1.0f / *wsum;
+    // this thread's share of the gradient: W2 rows 4 ty + i, columns 4 tx + j;
+    // W1 rows 4 ty + i, column tx; the vectors' entries 4 tx + j over the
+    // samples 4 ty + i of every tile
+    float gW2[4][4] = {}, gW1[4] = {}, gb1[4] = {}, gb2[4] = {}, gW3[4] = {}, gb3 = 0.f, lsum = 0.f;
+    const int ntiles = (n + kTile - 1) / kTile;
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int base = tile * kTile, rows = min(kTile, n - base);
+        __syncthreads();  // the last tile's reads, and the weights
+        for (int i = tid; i < kTile * kIn; i += kThreads) {
+            const int r = i / kIn, c = i % kIn;
+            const float v = r < rows ? X[(size_t)base * kIn + i] : 0.f;
+            s.Xri[r][c] = v;
+            s.Xir[c][r] = v;
+        }
+        if (tid < kTile) {
+            s.y[tid] = tid < rows ? y[base + tid] : 0.f;
+            s.w[tid] = tid < rows ? w[base + tid] * inv_w : 0.f;
+        }
+        __syncthreads();
+        // A1, H1: samples 4 ty + i, units 4 tx + j
+        {
+            float a[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) a[i][j] = s.b1[4 * tx + j];
+            outer4<kIn>(a, &s.Xir[0][0], 4 * ty, &s.W1ih[0][0], 4 * tx);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) a[i][j] = a[i][j] > 0.f ? a[i][j] : 0.f;
+            put4(&s.H1rh[0][0], &s.H1hr[0][0], a, 4 * ty, 4 * tx);
+        }
+        __syncthreads();
+        // A2, z, dz, D2
+        {
+            float a[4][4], w3[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) w3[j] = s.W3[4 * tx + j];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) a[i][j] = s.b2[4 * tx + j];
+            outer4<kH>(a, &s.H1hr[0][0], 4 * ty, &s.W2ho[0][0], 4 * tx);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int r = 4 * ty + i;
+                float p = 0.f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) p = fmaf(w3[j], a[i][j] > 0.f ? a[i][j] : 0.f, p);
+#pragma unroll
+                for (int o = 8; o >= 1; o >>= 1) p += __shfl_xor_sync(0xFFFFFFFFu, p, o);  // the 16 threads of a sample
+                const float z = p + b3, yy = s.y[r], ww = s.w[r];
+                const float dz = ww * (1.0f / (1.0f + expf(-z)) - yy);  // 0 for an absent sample (ww = 0)
+                if (tx == 0) {
+                    lsum += ww * (softplus(z) - yy * z);
+                    gb3 += dz;
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const bool on = a[i][j] > 0.f;
+                    const float d2 = on ? dz * w3[j] : 0.f;
+                    gW3[j] = fmaf(dz, on ? a[i][j] : 0.f, gW3[j]);
+                    gb2[j] += d2;
+                    a[i][j] = d2;
+                }
+            }
+            put4(&s.D2ro[0][0], &s.D2or[0][0], a, 4 * ty, 4 * tx);
+        }
+        __syncthreads();
+        outer4<kTile>(gW2, &s.D2ro[0][0], 4 * ty, &s.H1rh[0][0], 4 * tx);
+        // D1: samples 4 ty + i, units 4 tx + j
+        {
+            float a[4][4] = {};
+            outer4<kH>(a, &s.D2or[0][0], 4 * ty, &s.W2oh[0][0], 4 * tx);
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    a[i][j] = s.H1rh[4 * ty + i][4 * tx + j] > 0.f ? a[i][j] : 0.f;
+                    gb1[j] += a[i][j];
+                }
+            put4(&s.D1rh[0][0], nullptr, a, 4 * ty, 4 * tx);
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int r = 0; r < kTile; ++r) {
+            const float4 d1 = *reinterpret_cast<const float4 *>(&s.D1rh[r][4 * ty]);
+            const float x = s.Xri[r][tx];
+            gW1[0] = fmaf(d1.x, x, gW1[0]);
+            gW1[1] = fmaf(d1.y, x, gW1[1]);
+            gW1[2] = fmaf(d1.z, x, gW1[2]);
+            gW1[3] = fmaf(d1.w, x, gW1[3]);
+        }
+    }
+    const bool aligned = reinterpret_cast<uintptr_t>(G) % 16 == 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float *g2 = G + oW2 + (4 * ty + i) * kH + 4 * tx;
+        if (aligned) {
+            atomicAdd(reinterpret_cast<float4 *>(g2), make_float4(gW2[i][0], gW2[i][1], gW2[i][2], gW2[i][3]));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) atomicAdd(g2 + j, gW2[i][j]);
+        }
+        atomicAdd(&G[oW1 + (4 * ty + i) * kIn + tx], gW1[i]);
+    }
+    // the vectors: sums over ty through shared memory
+    __syncthreads();
+    float(*red)[3][kH] = reinterpret_cast<float(*)[3][kH]>(&s.H1hr[0][0]);  // [ty][vector][unit]
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        red[ty][0][4 * tx + j] = gb1[j];
+        red[ty][1][4 * tx + j] = gb2[j];
+        red[ty][2][4 * tx + j] = gW3[j];
+    }
+    if (tx == 0) {
+        s.y[ty] = lsum;
+        s.w[ty] = gb3;
     }
     __syncthreads();
-    // gW1 = D1^T X (64 x 16), gb1 = colsum D1
-    for (int i = tid; i < kH * kIn; i += kThreads) {
-        int o = i / kIn, c = i % kIn;
-        float g = 0.f;
-        for (int r = 0; r < kTile; ++r) g = fmaf(s.H1[r][o], s.X[r][c], g);
-        atomicAdd(&G[oW1 + i], g);
-    }
-    if (tid < kH) {
-        float g = 0.f;
-        for (int r = 0; r < kTile; ++r) g += s.H1[r][tid];
-        atomicAdd(&G[ob1 + tid], g);
+    if (tid < 3 * kH) {
+        const int v = tid / kH, u = tid % kH;
+        float t = 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) t += red[i][v][u];
+        atomicAdd(&G[(v == 0 ? ob1 : v == 1 ? ob2 : oW3) + u], t);
+    } else if (tid == 3 * kH) {
+        float t = 0.f;
+        for (int i = 0; i < 16; ++i) t += s.w[i];
+        atomicAdd(&G[ob3], t);
+    } else if (tid == 3 * kH + 32 && loss) {
+        float t = 0.f;
+        for (int i = 0; i < 16; ++i) t += s.y[i];
+        atomicAdd(loss, t);
     }
 }
 
@@ -209,10 +298,13 @@ extern "C" int sqg_mlp_grad(const float *params, const float *x, const float *y,
     const size_t smem = sizeof(TileSmem);
     if (cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return SQG_ERR_CUDA;
-    if (cudaMemsetAsync(grad, 0, sizeof(float) * SQG_MLP_NPARAM, stream) != cudaSuccess) return SQG_ERR_CUDA;
-    if (loss && cudaMemsetAsync(loss, 0, sizeof(float), stream) != cudaSuccess) return SQG_ERR_CUDA;
-    weight_sum_kernel<<<1, kThreads, 0, stream>>>(w, n, scratch);
-    mlp_grad_kernel<<<(n + kTile - 1) / kTile, kThreads, smem, stream>>>(params, x, y, w, n, scratch, grad, loss);
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return SQG_ERR_CUDA;
+    const int tiles = (n + kTile - 1) / kTile;  // one block per SM holds the tile buffers
+    prepare_kernel<<<1, kPrepThreads, 0, stream>>>(w, n, scratch, grad, loss);
+    mlp_grad_kernel<<<tiles < sms ? tiles : sms, kThreads, smem, stream>>>(params, x, y, w, n, scratch, grad, loss);
     return cudaGetLastError() == cudaSuccess ? SQG_OK : SQG_ERR_CUDA;
 }
 
