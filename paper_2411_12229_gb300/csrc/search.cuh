@@ -134,8 +134,9 @@ __device__ __forceinline__ bool mbar_try_wait_suspend(uint64_t *bar, uint32_t pa
 }
 // Bounded wait for phase `parity` of `bar`; false on timeout (never hangs).
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (__builtin_expect(mbar_try_wait(bar, parity), 1)) return true;
     const unsigned long long t0 = global_ns();
+#pragma unroll 1
     for (;;) {
         if (mbar_try_wait_suspend(bar, parity, 200000u)) return true;
         if (global_ns() - t0 > kWaitLimitNs) return false;
@@ -200,12 +201,15 @@ template <int T>
 __device__ __forceinline__ void hash_migrate(const uint32_t *S, uint32_t sbits, uint32_t *G, uint32_t gbits,
                                              const Team<T> &tm) {
     const uint32_t gsize = 1u << gbits, gmask = gsize - 1u;
+#pragma unroll 1
     for (uint32_t i = tm.tl; i < gsize; i += T) G[i] = kEmpty;
     tm.sync();
+#pragma unroll 1
     for (uint32_t i = tm.tl; i < (1u << sbits); i += T) {
         const uint32_t id = S[i];
         if (id == kEmpty) continue;
         uint32_t s = hslot(id, gbits);
+#pragma unroll 1
         while (atomicCAS(&G[s], kEmpty, id) != kEmpty) s = (s + 1) & gmask;
     }
     tm.sync();
@@ -213,6 +217,7 @@ __device__ __forceinline__ void hash_migrate(const uint32_t *S, uint32_t sbits, 
 __device__ __forceinline__ bool hash_contains(const uint32_t *H, uint32_t bits, uint32_t id) {
     const uint32_t mask = (1u << bits) - 1u;
     uint32_t s = hslot(id, bits);
+#pragma unroll 1
     for (;;) {
         uint32_t v = H[s];
         if (v == id) return true;
@@ -236,6 +241,7 @@ __device__ __forceinline__ QuerySide quantize_team(const float *qr, uint32_t d, 
     constexpr int V = Team<T>::V;
     const uint32_t nw = d / 32;
     float vl = __int_as_float(0x7f800000), vr = -vl;
+#pragma unroll 1
     for (uint32_t w = 0; w < nw; ++w) {
 #pragma unroll
         for (int v = 0; v < V; ++v) {
@@ -257,6 +263,7 @@ __device__ __forceinline__ QuerySide quantize_team(const float *qr, uint32_t d, 
     const float inv = range > 0.0f ? __fdiv_rn(15.0f, range) : 0.0f;
     qs.inv_sqrt_d = __fdiv_rn(1.0f, __fsqrt_rn((float)d));
     int sq = 0;
+#pragma unroll 1
     for (uint32_t w = 0; w < nw; ++w) {
         uint32_t b0 = 0, b1 = 0, b2 = 0, b3 = 0;
 #pragma unroll

@@ -77,6 +77,7 @@ __device__ __forceinline__ uint64_t shfl64_up(uint64_t v, int d) {
 __device__ __forceinline__ void hash_insert_warp(uint32_t *H, uint32_t bits, uint32_t id, int lane) {
     const uint32_t mask = (1u << bits) - 1u;
     uint32_t s = hslot(id, bits);
+#pragma unroll 1
     for (;;) {
         const uint32_t slot = (s + lane) & mask;
         const uint32_t emp = __ballot_sync(kFull, H[slot] == kEmpty);
@@ -224,21 +225,45 @@ __device__ __forceinline__ void exact_and_S(const float4 (&qv)[CH], const unsign
     }
 }
 
-// The key of neighbour j from its S (the estimator of Sec. 3.1.1 and the
-// bound-shifted key of reading R7), out-degree R: the same operations in
-// the same order as estimate_from_S.
+// The key of neighbour j (the estimator of Sec. 3.1.1 and the bound-shifted
+// key of reading R7), out-degree R, in two parts: what needs its S only, and
+// the rest from the vertex's exact distance.  The same operations in the same
+// order as estimate_from_S.
+struct EstPart {
+    float f_add, f_rescale, ip;
+};
 template <int R>
-__device__ __forceinline__ float keyR(const float *fac, const QuerySide &qs, uint32_t d, int j, int S, float dist_c,
-                                      float sqrt_dc, float eps0) {
-    const float f_add = fac[j], f_rescale = fac[R + j];
+__device__ __forceinline__ EstPart est_part(const float *fac, const QuerySide &qs, uint32_t d, int j, int S) {
+    EstPart e;
+    e.f_add = fac[j];
+    e.f_rescale = fac[R + j];
     const int pc = (int)reinterpret_cast<const uint32_t *>(fac)[3 * R + j];
     const float A = (float)(2 * S - qs.sq);
     const float B = __fmul_rn(qs.vl, (float)(2 * pc - (int)d));
-    const float ip = __fmul_rn(__fmaf_rn(qs.delta, A, B), qs.inv_sqrt_d);
-    const float est = __fmaf_rn(f_rescale, ip, __fadd_rn(f_add, dist_c));
+    e.ip = __fmul_rn(__fmaf_rn(qs.delta, A, B), qs.inv_sqrt_d);
+    return e;
+}
+template <int R>
+__device__ __forceinline__ float est_key(const EstPart &e, const float *fac, int j, float dist_c, float eps0) {
+    const float est = __fmaf_rn(e.f_rescale, e.ip, __fadd_rn(e.f_add, dist_c));
     if (eps0 == 0.0f) return est;
-    const float bound = __fmul_rn(fac[2 * R + j], sqrt_dc);
+    const float bound = __fmul_rn(fac[2 * R + j], __fsqrt_rn(dist_c));
     return __fsub_rn(est, __fmul_rn(eps0, bound));
+}
+
+// hash_contains from the value `v` of the id's first slot on.
+__device__ __forceinline__ bool hash_contains_from(uint32_t v, const uint32_t *H, uint32_t bits, uint32_t id) {
+    if (v == id) return true;
+    if (v == kEmpty) return false;
+    const uint32_t mask = (1u << bits) - 1u;
+    uint32_t s = hslot(id, bits);
+#pragma unroll 1
+    for (;;) {
+        s = (s + 1) & mask;
+        v = H[s];
+        if (v == id) return true;
+        if (v == kEmpty) return false;
+    }
 }
 
 // The key a packed entry holds (the inverse of key_bits; -0 comes back as +0).
@@ -272,6 +297,11 @@ __device__ __forceinline__ uint64_t pick(const uint64_t (&b)[NB], int s) {
 template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1>
 __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchArgs a) {
     using namespace compact;
+    // Up to this many admitted candidates are inserted one by one instead of
+    // merged (out-degree 32; 26 % of the expansions admit none, 30 % one or
+    // two): 45 warp-instructions each with two beam rows, against 140 for the
+    // merge's search, ranks and gather.
+    constexpr int kFew = NR == 1 ? (NB <= 4 ? 2 : 1) : 0;
     extern __shared__ __align__(128) unsigned char smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t d = a.d, nch = d / 4;
@@ -303,6 +333,7 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
         uint32_t status = 0;
         if (!(k >= 1 && k <= a.max_k && ef >= k && ef <= a.max_ef && (!a.uniform_k || k == a.uniform_k))) {
             const int kk = a.uniform_k ? a.uniform_k : (k < 0 ? 0 : (k > SQG_MAX_K ? SQG_MAX_K : k));
+#pragma unroll 1
             for (int t = lane; t < kk; t += 32) {
                 a.out_ids[off + t] = SQG_NO_ID;
                 a.out_dists[off + t] = __int_as_float(0x7f800000);
@@ -337,7 +368,9 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
         }
         uint32_t *H = Hs;
         uint32_t hbits = a.shash_bits;
-        for (uint32_t i = lane; i < (1u << hbits); i += 32) H[i] = kEmpty;
+#pragma unroll 1
+        for (uint32_t i = 4 * lane; i < (1u << hbits); i += 128)
+            *reinterpret_cast<uint4 *>(H + i) = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
 
         // ---- Algorithm 1, line 1: the beam holds the entry, which is expanded
         // first (its key, its exact distance, is set at that expansion)
@@ -370,7 +403,7 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
             *sst = StopCarry{0, 0.0f, 0.0f};
 
         for (;;) {
-            if (!mbar_wait_bounded(&bar[0], phase & 1u)) {
+            if (__builtin_expect(!mbar_wait_bounded(&bar[0], phase & 1u), 0)) {
                 status |= SQG_STATUS_TIMEOUT;
                 healthy = false;
                 break;
@@ -386,14 +419,67 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
 #pragma unroll
             for (int t = 0; t < NR; ++t) cid[t] = reinterpret_cast<const uint32_t *>(blk + a.off_ids)[lane + 32 * t];
             exact_and_S<CH, NR>(qv, blk, a.off_codes, planes, nch, d / 32, lane, dacc, S);
+            EstPart part[NR];
+            uint32_t hv[NR];  // each neighbour's first visited-set slot
+#pragma unroll
+            for (int t = 0; t < NR; ++t) {
+                part[t] = est_part<32 * NR>(reinterpret_cast<const float *>(blk + a.off_factors), qs, d, lane + 32 * t,
+                                            S[t]);
+                hv[t] = H[hslot(cid[t], hbits)];
+            }
             const float dist_c = exact_reduce<32>(dacc, tm);
-            if (hops == 1) {  // reading R8: the entry's key is its exact distance
+            // ---- line 5: the estimate and key of every neighbour from the same block
+            uint64_t cand[NR];
+            bool adm[NR];
+            uint32_t am[NR], anyam = 0;
+#pragma unroll
+            for (int t = 0; t < NR; ++t) {
+                const float key = est_key<32 * NR>(part[t], reinterpret_cast<const float *>(blk + a.off_factors),
+                                                   lane + 32 * t, dist_c, a.eps0);
+                cand[t] = pack_entry(key_bits(key), cid[t]);
+            }
+            if (__builtin_expect(hops == 1, 0)) {  // reading R8: the entry's key is its exact distance
                 if (lane == 0) {
                     b[0] = pack_entry(key_bits(dist_c), p) | 1ull;
                     beam_a[0] = b[0];
                 }
                 __syncwarp();
                 if (ef == 1) bworst = shfl64(b[0], 0);
+            }
+#pragma unroll
+            for (int t = 0; t < NR; ++t) {
+                // ---- line 6: unvisited neighbours enter the beam; an entry the
+                // cut to ef would drop at once is skipped early
+                adm[t] = cid[t] != kEmpty && cand[t] < bworst;
+                if (adm[t]) adm[t] = !hash_contains_from(hv[t], H, hbits, cid[t]);
+                am[t] = __ballot_sync(kFull, adm[t]);
+                anyam |= am[t];
+            }
+
+            // ---- lines 2-3 of the next step, taken now (Sec. 3.1.4: the next
+            // block is fetched while this step's merge runs): the next vertex
+            // is the smaller of the best admitted candidate and the first
+            // unvisited beam entry.  A candidate equal in (key, id) to a beam
+            // entry (dropped below as a duplicate) names that entry's vertex,
+            // which is unvisited, so it may stand in for it here.
+            uint64_t nxt;
+            {  // the smallest of the lane's admitted candidates and unvisited
+               // entries, then the warp's smallest (high word, then low word)
+                uint64_t v = kNone;
+#pragma unroll
+                for (int t = 0; t < NR; ++t) v = adm[t] && cand[t] < v ? cand[t] : v;
+#pragma unroll
+                for (int s = 0; s < NB; ++s) v = !(b[s] & 1ull) && b[s] < v ? b[s] : v;  // kNone: visited
+                const uint32_t chi = __reduce_min_sync(kFull, (uint32_t)(v >> 32));
+                const uint32_t clo = __reduce_min_sync(kFull, (uint32_t)(v >> 32) == chi ? (uint32_t)v : 0xFFFFFFFFu);
+                nxt = ((uint64_t)chi << 32) | clo;
+            }
+            const bool go = nxt != kNone && hops < hop_cap;  // a next expansion follows (the stop aside)
+            const uint32_t pn = entry_id(nxt);
+            __syncwarp();  // every lane's reads of the current block are done
+            if (go && lane == 0) {
+                fence_proxy_async();
+                bulk_fetch(buf, a.blocks + (size_t)pn * a.block_bytes, a.block_bytes, &bar[0]);
             }
             bool improved = false;
             {  // result top-k in registers: (dist bits << 32) | id, dist >= 0
@@ -421,43 +507,6 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
                     rworst = shfl64(pick<RK>(res, (k - 1) >> 5), (k - 1) & 31);
                 }
             }
-
-            // ---- line 5: the estimate and key of every neighbour from the same block
-            const float sqrt_dc = a.eps0 == 0.0f ? 0.0f : __fsqrt_rn(dist_c);
-            uint64_t cand[NR];
-            bool adm[NR];
-            uint32_t am[NR], anyam = 0;
-#pragma unroll
-            for (int t = 0; t < NR; ++t) {
-                const float key = keyR<32 * NR>(reinterpret_cast<const float *>(blk + a.off_factors), qs, d,
-                                                lane + 32 * t, S[t], dist_c, sqrt_dc, a.eps0);
-                cand[t] = pack_entry(key_bits(key), cid[t]);
-                // ---- line 6: unvisited neighbours enter the beam; an entry the
-                // cut to ef would drop at once is skipped early
-                adm[t] = cid[t] != kEmpty && cand[t] < bworst;
-                if (adm[t]) adm[t] = !hash_contains(H, hbits, cid[t]);
-                am[t] = __ballot_sync(kFull, adm[t]);
-                anyam |= am[t];
-            }
-
-            // ---- lines 2-3 of the next step, taken now (Sec. 3.1.4: the next
-            // block is fetched while this step's merge runs): the next vertex
-            // is the smaller of the best admitted candidate and the first
-            // unvisited beam entry.  A candidate equal in (key, id) to a beam
-            // entry (dropped below as a duplicate) names that entry's vertex,
-            // which is unvisited, so it may stand in for it here.
-            uint64_t nxt;
-            {  // the smallest of the lane's admitted candidates and unvisited
-               // entries, then the warp's smallest (high word, then low word)
-                uint64_t v = kNone;
-#pragma unroll
-                for (int t = 0; t < NR; ++t) v = adm[t] && cand[t] < v ? cand[t] : v;
-#pragma unroll
-                for (int s = 0; s < NB; ++s) v = !(b[s] & 1ull) && b[s] < v ? b[s] : v;  // kNone: visited
-                const uint32_t chi = __reduce_min_sync(kFull, (uint32_t)(v >> 32));
-                const uint32_t clo = __reduce_min_sync(kFull, (uint32_t)(v >> 32) == chi ? (uint32_t)v : 0xFFFFFFFFu);
-                nxt = ((uint64_t)chi << 32) | clo;
-            }
             if constexpr (!STOP) {  // (with the stop these two ends follow its decision)
                 if (nxt == kNone) break;  // no unvisited entry: the search ends (line 2)
                 if (hops >= hop_cap) {    // reading R6
@@ -465,19 +514,50 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
                     break;
                 }
             }
-            const bool go = !STOP || (nxt != kNone && hops < hop_cap);  // a next expansion follows
-            const uint32_t pn = entry_id(nxt);
-            __syncwarp();  // every lane's reads of the current block are done
-            if (go && lane == 0) {
-                fence_proxy_async();
-                bulk_fetch(buf, a.blocks + (size_t)pn * a.block_bytes, a.block_bytes, &bar[0]);
-            }
             int inserted = 0;  // this step's candidates kept by the cut (the stop's features)
 
             // ---- line 6: merge the admitted candidates, cut the beam to ef
             const uint64_t *B = beam_a;
             int pos[NR];
-            if (anyam) {
+            if (kFew > 0 && __popc(am[0]) <= kFew) {
+                if (anyam) {
+                    // a few candidates are inserted into the beam's registers one
+                    // by one: position by ballots, later entries up by shuffles
+                    int low = 32 * NB;
+                    bool entered = false;  // this lane's candidate
+#pragma unroll 1
+                    for (uint32_t left = am[0]; left; left &= left - 1) {
+                        const int src = __ffs(left) - 1;
+                        const uint64_t c = shfl64(cand[0], src);
+                        int at = 0;
+                        bool same = false;
+#pragma unroll
+                        for (int s = 0; s < NB; ++s) {
+                            at += __popc(__ballot_sync(kFull, b[s] < c));
+                            same |= ((b[s] ^ c) >> 1) == 0;
+                        }
+                        if (__any_sync(kFull, same) || at >= ef) continue;  // there already, or cut
+#pragma unroll
+                        for (int s = NB - 1; s >= 0; --s) {
+                            if (32 * s + 31 < at) continue;
+                            const uint64_t u = shfl64_up(b[s], 1);
+                            const uint64_t w = s > 0 ? shfl64(b[s > 0 ? s - 1 : 0], 31) : kNone;
+                            const int o = lane + 32 * s;
+                            if (o >= at) b[s] = o == at ? c : o >= ef ? kNone : lane == 0 ? w : u;
+                        }
+                        m = min(ef, m + 1);
+                        low = min(low, at);
+                        if (lane == src) entered = true;
+                    }
+#pragma unroll
+                    for (int s = 0; s < NB; ++s)
+                        if (32 * s + 31 >= low) beam_a[lane + 32 * s] = b[s];
+                    bworst = m == ef ? shfl64(pick<NB>(b, (ef - 1) >> 5), (ef - 1) & 31) : kNone;
+                    // (one that a smaller one pushed past the cut was not inserted)
+                    if constexpr (STOP) inserted = __popc(__ballot_sync(kFull, entered && cand[0] <= bworst));
+                }
+                anyam = 0;
+            } else if (anyam) {
                 anyam = 0;
 #pragma unroll
                 for (int t = 0; t < NR; ++t) {
@@ -509,7 +589,7 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
 #pragma unroll
                 for (int t = 0; t < NR; ++t) rank[t] = 0;
                 int j = 0;
-#pragma unroll 2
+#pragma unroll 1
                 for (; j + 2 <= nadm; j += 2) {  // two staged candidates per 16-byte read
                     const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(stage + j);
 #pragma unroll
@@ -663,7 +743,7 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
                 }
             hash_insert_warp(H, hbits, p, lane);  // its closing __syncwarp also orders the marks above
             ++hops;
-            if (Hg && H == Hs && (uint32_t)hops >= (1u << hbits) / 2) {
+            if (__builtin_expect(Hg && H == Hs && (uint32_t)hops >= (1u << hbits) / 2, 0)) {
                 hash_migrate<32>(Hs, hbits, Hg, a.hash_bits, tm);
                 H = Hg;
                 hbits = a.hash_bits;

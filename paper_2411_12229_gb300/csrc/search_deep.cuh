@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(128, MINB) search_deep_kernel(const SearchArgs
         uint32_t status = 0;
         if (!(k >= 1 && k <= a.max_k && ef >= k && ef <= a.max_ef && (!a.uniform_k || k == a.uniform_k))) {
             const int kk = a.uniform_k ? a.uniform_k : (k < 0 ? 0 : (k > SQG_MAX_K ? SQG_MAX_K : k));
+#pragma unroll 1
             for (int t = lane; t < kk; t += 32) {
                 a.out_ids[off + t] = SQG_NO_ID;
                 a.out_dists[off + t] = __int_as_float(0x7f800000);
@@ -142,7 +143,9 @@ __global__ void __launch_bounds__(128, MINB) search_deep_kernel(const SearchArgs
         }
         uint32_t *H = Hs;
         uint32_t hbits = a.shash_bits;
-        for (uint32_t i = lane; i < (1u << hbits); i += 32) H[i] = kEmpty;
+#pragma unroll 1
+        for (uint32_t i = 4 * lane; i < (1u << hbits); i += 128)
+            *reinterpret_cast<uint4 *>(H + i) = make_uint4(kEmpty, kEmpty, kEmpty, kEmpty);
 
         // ---- Algorithm 1, line 1: the beam holds the entry, which is expanded
         // first (its key, its exact distance, is set at that expansion)
@@ -201,7 +204,26 @@ __global__ void __launch_bounds__(128, MINB) search_deep_kernel(const SearchArgs
 #pragma unroll
             for (int t = 0; t < NR; ++t) cid[t] = reinterpret_cast<const uint32_t *>(blk + a.off_ids)[lane + 32 * t];
             exact_and_S<CH, NR>(qv, blk, a.off_codes, planes, nch, d / 32, lane, dacc, S);
+            EstPart part[NR];
+            uint32_t hv[NR];  // each neighbour's first visited-set slot
+#pragma unroll
+            for (int t = 0; t < NR; ++t) {
+                part[t] = est_part<32 * NR>(reinterpret_cast<const float *>(blk + a.off_factors), qs, d, lane + 32 * t,
+                                            S[t]);
+                hv[t] = H[hslot(cid[t], hbits)];
+            }
             const float dist_c = exact_reduce<32>(dacc, tm);
+            // ---- line 5: the estimate and key of every neighbour from the same block
+            uint64_t cand[NR];
+            bool adm[NR];
+            uint32_t am[NR];
+            int nadm = 0;
+#pragma unroll
+            for (int t = 0; t < NR; ++t) {
+                const float key = est_key<32 * NR>(part[t], reinterpret_cast<const float *>(blk + a.off_factors),
+                                                   lane + 32 * t, dist_c, a.eps0);
+                cand[t] = pack_entry(key_bits(key), cid[t]);
+            }
             if (hops == 1) {  // reading R8: the entry's key is its exact distance
                 if (lane == 0) {
                     b[0] = pack_entry(key_bits(dist_c), p) | 1ull;
@@ -209,6 +231,36 @@ __global__ void __launch_bounds__(128, MINB) search_deep_kernel(const SearchArgs
                 }
                 __syncwarp();
                 if (ef == 1) bworst = shfl64(b[0], 0);
+            }
+#pragma unroll
+            for (int t = 0; t < NR; ++t) {
+                // ---- line 6: unvisited neighbours enter the beam; an entry the
+                // cut to ef would drop at once is skipped early
+                adm[t] = cid[t] != kEmpty && cand[t] < bworst;
+                if (adm[t]) adm[t] = !hash_contains_from(hv[t], H, hbits, cid[t]);
+                am[t] = __ballot_sync(kFull, adm[t]);
+                nadm += __popc(am[t]);
+            }
+
+            // ---- lines 2-3 of the next step: the smallest unvisited entry of
+            // candidates, front and window
+            uint64_t v = win & 1ull ? kNone : win;
+#pragma unroll
+            for (int t = 0; t < NR; ++t) v = adm[t] && cand[t] < v ? cand[t] : v;
+#pragma unroll
+            for (int s = 0; s < NB; ++s) v = !(b[s] & 1ull) && b[s] < v ? b[s] : v;  // kNone: visited
+            uint64_t nxt = warp_min64(v);
+            bool late = false;  // nxt may be past the cut: choose after a full merge
+            if (!shallow && nxt != kNone && wbase + 32 + mf >= ef) {
+                int smaller = wbase + __popc(__ballot_sync(kFull, win < nxt));
+#pragma unroll
+                for (int s = 0; s < NB; ++s) smaller += __popc(__ballot_sync(kFull, b[s] < nxt));
+                late = smaller >= ef;
+            }
+            __syncwarp();  // every lane's reads of the current block are done
+            if (nxt != kNone && !late && hops < hop_cap && lane == 0) {
+                fence_proxy_async();
+                bulk_fetch(buf, a.blocks + (size_t)entry_id(nxt) * a.block_bytes, a.block_bytes, &bar[0]);
             }
             {  // result top-k in registers: (dist bits << 32) | id, dist >= 0
                 const uint64_t r = ((uint64_t)__float_as_uint(dist_c) << 32) | p;
@@ -232,52 +284,10 @@ __global__ void __launch_bounds__(128, MINB) search_deep_kernel(const SearchArgs
                     rworst = shfl64(pick<RK>(res, (k - 1) >> 5), (k - 1) & 31);
                 }
             }
-
-            // ---- line 5: the estimate and key of every neighbour from the same block
-            const float sqrt_dc = a.eps0 == 0.0f ? 0.0f : __fsqrt_rn(dist_c);
-            uint64_t cand[NR];
-            bool adm[NR];
-            uint32_t am[NR];
-            int nadm = 0;
-#pragma unroll
-            for (int t = 0; t < NR; ++t) {
-                const float key = keyR<32 * NR>(reinterpret_cast<const float *>(blk + a.off_factors), qs, d,
-                                                lane + 32 * t, S[t], dist_c, sqrt_dc, a.eps0);
-                cand[t] = pack_entry(key_bits(key), cid[t]);
-                // ---- line 6: unvisited neighbours enter the beam; an entry the
-                // cut to ef would drop at once is skipped early
-                adm[t] = cid[t] != kEmpty && cand[t] < bworst;
-                if (adm[t]) adm[t] = !hash_contains(H, hbits, cid[t]);
-                am[t] = __ballot_sync(kFull, adm[t]);
-                nadm += __popc(am[t]);
-            }
-
-            // ---- lines 2-3 of the next step: the smallest unvisited entry of
-            // candidates, front and window
-            uint64_t v = win & 1ull ? kNone : win;
-#pragma unroll
-            for (int t = 0; t < NR; ++t) v = adm[t] && cand[t] < v ? cand[t] : v;
-#pragma unroll
-            for (int s = 0; s < NB; ++s) v = !(b[s] & 1ull) && b[s] < v ? b[s] : v;  // kNone: visited
-            uint64_t nxt = warp_min64(v);
             if (nxt == kNone) break;  // no unvisited entry: the search ends (line 2)
-            bool late = false;        // nxt may be past the cut: choose after a full merge
-            if (!shallow && wbase + 32 + mf >= ef) {
-                int smaller = wbase + __popc(__ballot_sync(kFull, win < nxt));
-#pragma unroll
-                for (int s = 0; s < NB; ++s) smaller += __popc(__ballot_sync(kFull, b[s] < nxt));
-                late = smaller >= ef;
-            }
-            __syncwarp();  // every lane's reads of the current block are done
-            if (!late) {
-                if (hops >= hop_cap) {  // reading R6
-                    status |= SQG_STATUS_CAPACITY;
-                    break;
-                }
-                if (lane == 0) {
-                    fence_proxy_async();
-                    bulk_fetch(buf, a.blocks + (size_t)entry_id(nxt) * a.block_bytes, a.block_bytes, &bar[0]);
-                }
+            if (!late && hops >= hop_cap) {  // reading R6
+                status |= SQG_STATUS_CAPACITY;
+                break;
             }
 
             // ---- line 6: step 0 merges the candidates into the front (the
