@@ -78,6 +78,7 @@ struct SearchArgs {
     int path_cap;
     uint32_t warp_bytes, cta_bytes;
     uint32_t o_buf0, o_buf1, o_bar, o_beam, o_hash, o_res, o_planes, o_spos;
+    uint32_t o_log;  // the compact kernel's result log (more than 32 results, no stop)
 };
 
 // ---------------------------------------------------------------- PTX helpers

@@ -15,9 +15,10 @@
 
 #include "../../include/sqg.h"
 #include "index_format.h"
-#include "search.cuh"
+#include "search_compact.cuh"
 
 using namespace sqg;
+using sqg::compact::kLogSize;
 
 struct sqg_index {
     int device;
@@ -464,6 +465,8 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
         // hidden values between its layers
         a.o_spos = (uint32_t)o; o = align_up(o + std::max<size_t>(4 * (size_t)R, 256), 16);
     }
+    a.o_log = (uint32_t)o;
+    if (pl.compact && pl.crk > 1 && !p.stop_mlp) o += 8 * (size_t)kLogSize;
     // visited set: up to 2^10 slots in shared memory; a longer search moves
     // to its warp's full-size table in the workspace
     const uint32_t smem_bits_default = 9u;  // 2^10 measured slower at large beams (less residency)
