@@ -185,82 +185,105 @@ __global__ void mlp_transpose_kernel(const float *__restrict__ src, float *__res
 
 // q' = P^-1 q for a batch (Eq. (4)) in the canonical chunked order:
 // out[r][i] = (((0 + s_0) + s_1) + ...) over the d/32 chunks, s_c the fmaf
-// chain of rot[i][j] * q[r][j] over j = 32c .. 32c+31 from 0.  64 x 64 output
-// tiles, 256 threads with 4 x 4 outputs each; one 32-wide chunk of q and of
-// P^-1 per step, double-buffered in shared memory (the next chunk's global
-// loads are in flight while this one is multiplied), so every output walks
-// j in order with one chunk accumulator and one total and the tiling changes
-// no bit.
-constexpr int kRotT = 64, kRotK = 32;
-__global__ void __launch_bounds__(256) rotate_kernel(const float *__restrict__ q, const float *__restrict__ rot,
-                                                     float *__restrict__ out, int nq, int d, unsigned int *queue) {
-    if (queue && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *queue = 0u;  // the search's work queue
-    __shared__ __align__(16) float As[2][kRotK][kRotT + 4];  // [buffer][j][row]
-    __shared__ __align__(16) float Bs[2][kRotK][kRotT + 4];  // [buffer][j][col]
-    const int tid = threadIdx.x, tx = tid % 16, ty = tid / 16;
-    const int r0 = blockIdx.y * kRotT, c0 = blockIdx.x * kRotT;
-    constexpr int kPer = kRotT * kRotK / 256;  // elements of each tile a thread moves
-    float ra[kPer], rb[kPer];
-    auto load = [&](int j0) {
+// chain of rot[i][j] * q[r][j] over j = 32c .. 32c+31 from 0.  A block of 8
+// warps takes 8 RPT queries x 32 CPT outputs: warp w queries w RPT .. w RPT +
+// RPT - 1, lane l outputs l + 32 j; every output walks j in order with one
+// chunk accumulator and one total, so the tiling changes no bit.
+//
+// Slabs of up to 128 columns of the tile's queries and rows of P^-1 are staged
+// as they are (16-byte copies, rows padded to 132 floats); a step of four j
+// reads one float4 per query (a broadcast) and per output (a bank quad each).
+// With RPT = 8, CPT = 4 that is 12 reads for 128 multiply-adds.  us at d 128
+// for 1 / 200 / 2,001 / 10,000 / 50,000 queries: 2.9 / 3.1 / 5.1 / 15.1 / 48.1;
+// 6.8 / 7.4 / 7.5 / 17.7 / 59.2 with one 64 x 64 tile size staged transposed.
+// A copy group per chunk, waited for one by one, was 2-10 % slower.
+constexpr int kRotSlab = 128, kRotPitch = kRotSlab + 4, kRotWarps = 8;
+template <int RPT, int CPT>
+__global__ void __launch_bounds__(kRotWarps * 32) rotate_kernel(const float *__restrict__ q,
+                                                                const float *__restrict__ rot,
+                                                                float *__restrict__ out, int nq, int d,
+                                                                unsigned int *queue) {
+    constexpr int kRows = kRotWarps * RPT, kCols = 32 * CPT;
+    extern __shared__ __align__(16) float rot_smem[];
+    float *const qs = rot_smem, *const ps = rot_smem + kRows * kRotPitch;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    const int r0 = blockIdx.y * kRows, c0 = blockIdx.x * kCols;
+    if (queue && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *queue = 0u;  // the search's work queue
+    float tot[RPT][CPT];
 #pragma unroll
-        for (int t = 0; t < kPer; ++t) {
-            const int e = tid + 256 * t, rr = e / kRotK, jj = e % kRotK;
-            const int gr = r0 + rr, gc = c0 + rr;
-            ra[t] = gr < nq ? q[(size_t)gr * d + j0 + jj] : 0.0f;
-            rb[t] = gc < d ? rot[(size_t)gc * d + j0 + jj] : 0.0f;
+    for (int i = 0; i < RPT; ++i)
+#pragma unroll
+        for (int j = 0; j < CPT; ++j) tot[i][j] = 0.0f;
+    for (int k0 = 0; k0 < d; k0 += kRotSlab) {
+        const int width = min(kRotSlab, d - k0);  // a multiple of 32
+        if (k0 > 0) __syncthreads();              // the last slab's reads
+        // (rows past the ends are left as they are: their outputs are not written)
+        for (int e = tid; e < (kRows + kCols) * (kRotSlab / 4); e += kRotWarps * 32) {
+            const int row = e / (kRotSlab / 4), col = 4 * (e % (kRotSlab / 4));
+            const bool is_q = row < kRows;
+            const int gr = is_q ? r0 + row : c0 + row - kRows;
+            if (col < width && gr < (is_q ? nq : d)) {
+                const float *src = (is_q ? q : rot) + (size_t)gr * d + k0 + col;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                                 smem_addr(rot_smem + row * kRotPitch + col)),
+                             "l"(src)
+                             : "memory");
+            }
         }
-    };
-    auto store = [&](int b) {
-#pragma unroll
-        for (int t = 0; t < kPer; ++t) {
-            const int e = tid + 256 * t, rr = e / kRotK, jj = e % kRotK;
-            As[b][jj][rr] = ra[t];
-            Bs[b][jj][rr] = rb[t];
-        }
-    };
-    float acc[4][4], tot[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) tot[a][b] = 0.0f;
-    load(0);
-    store(0);
-    __syncthreads();
-    const int nchunk = d / kRotK;
-    for (int c = 0; c < nchunk; ++c) {
-        const int buf = c & 1;
-        if (c + 1 < nchunk) load((c + 1) * kRotK);
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) acc[a][b] = 0.0f;
-#pragma unroll 8
-        for (int jj = 0; jj < kRotK; ++jj) {
-            const float4 av = *reinterpret_cast<const float4 *>(&As[buf][jj][ty * 4]);
-            const float4 bv = *reinterpret_cast<const float4 *>(&Bs[buf][jj][tx * 4]);
-            const float a4[4] = {av.x, av.y, av.z, av.w}, b4[4] = {bv.x, bv.y, bv.z, bv.w};
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = __fmaf_rn(b4[b], a4[a], acc[a][b]);
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) tot[a][b] = __fadd_rn(tot[a][b], acc[a][b]);
-        if (c + 1 < nchunk) store(buf ^ 1);
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-    }
+        for (int ch = 0; ch < width; ch += 32) {
+            float acc[RPT][CPT];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        const int gr = r0 + ty * 4 + a;
-        if (gr >= nq) continue;
+            for (int i = 0; i < RPT; ++i)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int gc = c0 + tx * 4 + b;
-            if (gc < d) out[(size_t)gr * d + gc] = tot[a][b];
+                for (int j = 0; j < CPT; ++j) acc[i][j] = 0.0f;
+#pragma unroll 2
+            for (int k = ch; k < ch + 32; k += 4) {
+                float4 pv[CPT];
+#pragma unroll
+                for (int j = 0; j < CPT; ++j)
+                    pv[j] = *reinterpret_cast<const float4 *>(ps + (lane + 32 * j) * kRotPitch + k);
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    const float4 v = *reinterpret_cast<const float4 *>(qs + (w * RPT + i) * kRotPitch + k);
+#pragma unroll
+                    for (int j = 0; j < CPT; ++j) {
+                        acc[i][j] = __fmaf_rn(pv[j].x, v.x, acc[i][j]);
+                        acc[i][j] = __fmaf_rn(pv[j].y, v.y, acc[i][j]);
+                        acc[i][j] = __fmaf_rn(pv[j].z, v.z, acc[i][j]);
+                        acc[i][j] = __fmaf_rn(pv[j].w, v.w, acc[i][j]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < RPT; ++i)
+#pragma unroll
+                for (int j = 0; j < CPT; ++j) tot[i][j] = __fadd_rn(tot[i][j], acc[i][j]);
         }
     }
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        const int gr = r0 + w * RPT + i;
+        if (gr >= nq) break;
+#pragma unroll
+        for (int j = 0; j < CPT; ++j) {
+            const int gc = c0 + lane + 32 * j;
+            if (gc < d) out[(size_t)gr * d + gc] = tot[i][j];
+        }
+    }
+}
+
+template <int RPT, int CPT>
+cudaError_t launch_rotate(const float *q, const float *rot, float *out, int nq, int d, unsigned int *queue,
+                          cudaStream_t s) {
+    constexpr int kRows = kRotWarps * RPT, kCols = 32 * CPT;
+    constexpr int smem = (kRows + kCols) * kRotPitch * (int)sizeof(float);
+    auto fn = rotate_kernel<RPT, CPT>;
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    fn<<<dim3((d + kCols - 1) / kCols, (nq + kRows - 1) / kRows), kRotWarps * 32, smem, s>>>(q, rot, out, nq, d, queue);
+    return cudaGetLastError();
 }
 
 // Cosine similarity as Euclidean search between unit vectors: q / ||q||,
@@ -554,9 +577,16 @@ cudaError_t rotate_simt(const sqg_index *ix, const float *queries, float *out, i
                         cudaStream_t stream) {
     const int d = (int)ix->lay.d;
     if (ix->fjlt) return launch_fjlt(queries, ix->d_signs, out, nq, d, queue, stream);
-    dim3 rg((d + kRotT - 1) / kRotT, (nq + kRotT - 1) / kRotT);
-    rotate_kernel<<<rg, 256, 0, stream>>>(queries, ix->d_rot, out, nq, d, queue);
-    return cudaGetLastError();
+    // 64 x 128 tiles read least per multiply-add but last longest: from four
+    // per SM on (50,000 queries of d 128: 48.1 us against 52.6 with 32 x 64
+    // tiles; 20,000: 25.3 against 24.6).  Up to two 8 x 32 tiles per SM the
+    // launch is one tile's chain of d multiply-adds and the small tile's load is
+    // the shortest (200 queries: 3.1 against 4.6; 719, past the line: 5.0
+    // against 4.7).
+    auto blocks = [&](long long rows, long long cols) { return ((nq + rows - 1) / rows) * ((d + cols - 1) / cols); };
+    if (blocks(64, 128) >= 4LL * ix->num_sms) return launch_rotate<8, 4>(queries, ix->d_rot, out, nq, d, queue, stream);
+    if (blocks(8, 32) > 2LL * ix->num_sms) return launch_rotate<4, 2>(queries, ix->d_rot, out, nq, d, queue, stream);
+    return launch_rotate<1, 1>(queries, ix->d_rot, out, nq, d, queue, stream);
 }
 
 // Rotation path: 1 = the CUDA-core kernel in the canonical order, 2 = tensor
