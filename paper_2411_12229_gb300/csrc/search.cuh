@@ -1015,8 +1015,8 @@ __global__ void __launch_bounds__(128, (LEAN ? 8 : (CH <= 2 ? 5 : 3))) search_ke
     }
 }
 
-// sqg_workspace_size, with or without the deep-beam kernel's own needs (sqg_api.cu).
-size_t workspace_need(const sqg_index *ix, int nq, int max_k, int max_ef, bool allow_deep);
+// sqg_workspace_size, or (generous false) the least workspace a search accepts (sqg_api.cu).
+size_t workspace_need(const sqg_index *ix, int nq, int max_k, int max_ef, bool generous);
 
 // Host-side launch helpers, defined in the instantiation units.
 // Tensor-core rotation and the exact quantization after it (rotate_tc.cu).

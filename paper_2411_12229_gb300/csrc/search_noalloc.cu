@@ -35,7 +35,7 @@
 #include "../../include/sqg.h"
 
 namespace sqg {
-size_t workspace_need(const sqg_index *ix, int nq, int max_k, int max_ef, bool allow_deep);  // sqg_api.cu
+size_t workspace_need(const sqg_index *ix, int nq, int max_k, int max_ef, bool generous);  // sqg_api.cu
 }
 
 namespace {

@@ -153,7 +153,8 @@ __global__ void plan_kernel(const int32_t *k, const int32_t *ef, int nq, long lo
 __global__ void mlp_transpose_kernel(const float *__restrict__ src, float *__restrict__ dst) {
     const float *W1 = src, *b1 = W1 + 64 * SQG_MLP_IN, *W2 = b1 + 64, *b2 = W2 + 64 * 64, *W3 = b2 + 64;
     float *t = dst;
-    for (int e = threadIdx.x; e < 8 * 32; e += blockDim.x) {  // W1p[i2][l]
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, step = gridDim.x * blockDim.x;
+    for (int e = tid; e < 8 * 32; e += step) {  // W1p[i2][l]
         const int i2 = e / 32, l = e % 32;
         t[4 * e + 0] = W1[l * SQG_MLP_IN + 2 * i2];
         t[4 * e + 1] = W1[(l + 32) * SQG_MLP_IN + 2 * i2];
@@ -161,12 +162,12 @@ __global__ void mlp_transpose_kernel(const float *__restrict__ src, float *__res
         t[4 * e + 3] = W1[(l + 32) * SQG_MLP_IN + 2 * i2 + 1];
     }
     t += 8 * 32 * 4;
-    for (int l = threadIdx.x; l < 32; l += blockDim.x) {
+    for (int l = tid; l < 32; l += step) {
         t[2 * l] = b1[l];
         t[2 * l + 1] = b1[l + 32];
     }
     t += 64;
-    for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {  // W2p[i2][l]
+    for (int e = tid; e < 32 * 32; e += step) {  // W2p[i2][l]
         const int i2 = e / 32, l = e % 32;
         t[4 * e + 0] = W2[l * 64 + 2 * i2];
         t[4 * e + 1] = W2[(l + 32) * 64 + 2 * i2];
@@ -174,13 +175,13 @@ __global__ void mlp_transpose_kernel(const float *__restrict__ src, float *__res
         t[4 * e + 3] = W2[(l + 32) * 64 + 2 * i2 + 1];
     }
     t += 32 * 32 * 4;
-    for (int l = threadIdx.x; l < 32; l += blockDim.x) {
+    for (int l = tid; l < 32; l += step) {
         t[2 * l] = b2[l];
         t[2 * l + 1] = b2[l + 32];
         t[64 + 2 * l] = W3[l];
         t[64 + 2 * l + 1] = W3[l + 32];
     }
-    if (threadIdx.x == 0) t[128] = W3[64];  // b3
+    if (tid == 0) t[128] = W3[64];  // b3
 }
 
 // q' = P^-1 q for a batch (Eq. (4)) in the canonical chunked order:
@@ -417,7 +418,9 @@ struct LaunchPlan {
 enum Trace { kNoTrace, kTracePath, kTraceFeatures };
 
 int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_search_params &p, LaunchPlan &pl,
-              Trace traced = kNoTrace, bool allow_deep = true) {
+              Trace traced = kNoTrace, bool generous = true) {
+    // generous false: the general kernel where the compact one does not apply, the
+    // smaller visited tables -- the least workspace
     const uint32_t d = ix->lay.d, R = ix->lay.R, bb = ix->lay.block_bytes;
     pl.ch = pick_ch(d);
     pl.nb = (int)(R / 32);
@@ -437,7 +440,7 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
     // 5.08 / 3.12, ef 800 10.7 / 5.15.  Within the compact kernel's range the
     // two are within 8 % at ef 129-256 and the compact one is faster below (ef
     // 64: 0.36 / 0.42; d 960 ef 112: 2.55 / 2.72).
-    pl.deep = allow_deep && !pl.compact && p.kernel == 0 && pl.team == 32 && max_k <= 128 && p.multi_estimate && !p.stop_mlp &&
+    pl.deep = generous && !pl.compact && p.kernel == 0 && pl.team == 32 && max_k <= 128 && p.multi_estimate && !p.stop_mlp &&
               traced != kTraceFeatures && p.prefetch != 2 && p.lean != 2;
     pl.cbnb = max_ef <= 64 ? 2 : max_ef <= 128 ? 4 : 8;
     pl.crk = max_k <= 32 ? 1 : 4;
@@ -490,15 +493,17 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
     }
     a.o_log = (uint32_t)o;
     if (pl.compact && pl.crk > 1 && !p.stop_mlp) o += 8 * (size_t)kLogSize;
-    // visited set: up to 2^10 slots in shared memory; a longer search moves
-    // to its warp's full-size table in the workspace
-    const uint32_t smem_bits_default = 9u;  // 2^10 measured slower at large beams (less residency)
-    a.shash_bits =
-        std::min<uint32_t>(bits, p.visited_smem_log2 > 0 ? (uint32_t)p.visited_smem_log2 : smem_bits_default);
-    pl.ghash = a.shash_bits < bits;
+    // visited set: 2^9 slots in shared memory (more cost resident warps: 2^10
+    // is 9 % slower for 16,384 candidate searches at ef 400); a search past
+    // half of them moves to its warp's full-size table in the workspace.  A
+    // batch whose queries are all resident at once has no use for more warps:
+    // it takes up to 2^11 slots, which spares it the move and the global probes
+    // (719 queries of d 96: ef 160 492 -> 463 us, ef 400 1,074 -> 1,016; 500 of
+    // d 1536 at ef 400 1,567 -> 1,536).
     a.o_hash = (uint32_t)o;
-    const size_t warp_bytes = align_up(o + ((size_t)4 << a.shash_bits), 128);
     const size_t cta = 0;  // the stop network's weights are read from the workspace (L1-cached)
+    size_t warp_bytes = 0;
+    int warps = 0, per_sm = 0;
     // one slot of warp_bytes per query in flight: V per warp
     auto occupancy = [&](int w, int *blocks) -> cudaError_t {
         const size_t sm = cta + (size_t)w * V * warp_bytes;
@@ -513,12 +518,15 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
              : pl.nb == 1   ? search_occupancy_nb1(pl.ch, w * 32, sm, blocks)
                             : search_occupancy_nb2(pl.ch, w * 32, sm, blocks);
     };
-    int warps = 0, per_sm = 0;
-    if (p.warps_per_block > 0) {
-        warps = std::min(p.warps_per_block, 4);
-        while (warps > 1 && cta + warps * V * warp_bytes > ix->smem_optin) --warps;
-        if (occupancy(warps, &per_sm) != cudaSuccess) return SQG_ERR_CUDA;
-    } else {
+    auto residency = [&](uint32_t slots_log2) -> int {
+        a.shash_bits = std::min<uint32_t>(bits, slots_log2);
+        warp_bytes = align_up(o + ((size_t)4 << a.shash_bits), 128);
+        warps = per_sm = 0;
+        if (p.warps_per_block > 0) {
+            warps = std::min(p.warps_per_block, 4);
+            while (warps > 1 && cta + warps * V * warp_bytes > ix->smem_optin) --warps;
+            return occupancy(warps, &per_sm) == cudaSuccess ? SQG_OK : SQG_ERR_CUDA;
+        }
         // the block size with the most resident warps per SM (shared memory
         // limits large d, registers small d); larger blocks on a tie
         for (int w : {4, 2, 1}) {
@@ -529,7 +537,18 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
                 per_sm = b;
             }
         }
-    }
+        return SQG_OK;
+    };
+    bool sized = false;
+    if (p.visited_smem_log2 == 0 && (pl.compact || pl.deep) && generous && bits > 9)
+        for (uint32_t b : {11u, 10u}) {
+            if (sized || (b == 11u && bits < 11u)) continue;
+            if (residency(b) != SQG_OK) return SQG_ERR_CUDA;
+            sized = (long long)per_sm * warps * ix->num_sms >= nq;
+        }
+    if (!sized && residency(p.visited_smem_log2 > 0 ? (uint32_t)p.visited_smem_log2 : 9u) != SQG_OK)
+        return SQG_ERR_CUDA;
+    pl.ghash = a.shash_bits < bits;
     if (warps < 1 || per_sm < 1) return SQG_ERR_CAPACITY;
     a.warp_bytes = (uint32_t)warp_bytes;
     a.cta_bytes = (uint32_t)cta;
@@ -802,20 +821,20 @@ extern "C" int sqg_index_info(const sqg_index *ix, sqg_info *out) {
     return SQG_OK;
 }
 
-size_t sqg::workspace_need(const sqg_index *ix, int nq, int max_k, int max_ef, bool allow_deep) {
+size_t sqg::workspace_need(const sqg_index *ix, int nq, int max_k, int max_ef, bool generous) {
     if (!ix || nq < 0 || max_k < 1 || max_k > SQG_MAX_K || max_ef < max_k || max_ef > SQG_MAX_EF) return 0;
     DeviceGuard g(ix->device);
     // the larger of the plans without and with the learned stop's weights
     LaunchPlan pl;
     sqg_search_params p = default_params();
-    if (make_plan(ix, nq, max_k, max_ef, p, pl, kNoTrace, allow_deep) != SQG_OK) return 0;
+    if (make_plan(ix, nq, max_k, max_ef, p, pl, kNoTrace, generous) != SQG_OK) return 0;
     size_t need = pl.ws_total;
     p.kernel = 1;  // the general kernel (its visited tables follow its own residency)
-    if (make_plan(ix, nq, max_k, max_ef, p, pl) == SQG_OK) need = std::max(need, pl.ws_total);
+    if (make_plan(ix, nq, max_k, max_ef, p, pl, kNoTrace, generous) == SQG_OK) need = std::max(need, pl.ws_total);
     p.stop_mlp = reinterpret_cast<const float *>(16);  // any non-null: only the layout is planned
-    if (make_plan(ix, nq, max_k, max_ef, p, pl) == SQG_OK) need = std::max(need, pl.ws_total);
+    if (make_plan(ix, nq, max_k, max_ef, p, pl, kNoTrace, generous) == SQG_OK) need = std::max(need, pl.ws_total);
     p.kernel = 0;  // the compact kernel's build with the stop fused
-    if (make_plan(ix, nq, max_k, max_ef, p, pl) == SQG_OK) need = std::max(need, pl.ws_total);
+    if (make_plan(ix, nq, max_k, max_ef, p, pl, kNoTrace, generous) == SQG_OK) need = std::max(need, pl.ws_total);
     return need;
 }
 
@@ -872,9 +891,8 @@ static int search_impl(const sqg_index *ix, const float *queries, int nq, const 
     LaunchPlan pl;
     const Trace traced = trace_feat || trace_n ? kTraceFeatures : path ? kTracePath : kNoTrace;
     int rc = make_plan(ix, nq, max_k, max_ef, p, pl, traced);
-    // more resident warps need more visited tables: a workspace that holds
-    // the general kernel's still serves
-    if (rc == SQG_OK && pl.deep && workspace && ws_bytes < pl.ws_total)
+    // a workspace that holds the least plan's tables still serves
+    if (rc == SQG_OK && workspace && ws_bytes < pl.ws_total)
         rc = make_plan(ix, nq, max_k, max_ef, p, pl, traced, false);
     if (rc != SQG_OK) return rc;
     bool own_ws = false;
@@ -920,7 +938,7 @@ static int search_impl(const sqg_index *ix, const float *queries, int nq, const 
     a.mlp = nullptr;
     if (p.stop_mlp) {
         float *t = reinterpret_cast<float *>(ws + pl.ws_mlp);
-        mlp_transpose_kernel<<<1, 256, 0, stream>>>(p.stop_mlp, t);
+        mlp_transpose_kernel<<<16, 64, 0, stream>>>(p.stop_mlp, t);  // one element a thread: 7 -> 2 us
         a.mlp = t;
     }
     a.stop_logit = p.stop_logit;

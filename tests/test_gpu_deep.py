@@ -106,3 +106,45 @@ def test_deep_mixed_batch(gpu_tiny):
     a = ix.search(qd, kt, et, stats=True, max_k=100, max_ef=800)
     b = ix.search(qd, kt, et, stats=True, max_k=100, max_ef=800, kernel=1)
     assert same(a, b)
+
+
+def test_least_workspace_still_serves(tmp_path, lib_built):
+    """A workspace (or the fixed scratch) that holds the general kernel's
+    visited tables but not the deep kernel's, whose build for d <= 512 keeps
+    more warps resident: the search takes the general kernel, not an error."""
+    from paper_2411_12229_gb300 import _binding as B
+    from paper_2411_12229_gb300 import index_builder as ib
+    from paper_2411_12229_gb300 import synth
+    from paper_2411_12229_gb300.api import Index
+    w = synth.small(synth.HIGHDIM_1M_D960.with_(d=512), 1500, 2400)
+    p = tmp_path / "d512.sqg"
+    ib.build_index(p, synth.base(w), 32)
+    ix, q = Index(p, 0), torch.from_numpy(synth.queries(w)).cuda()
+    k, ef, nq = 10, 300, q.shape[0]
+    least, full = ix.workspace_size(nq, k, ef, kernel=1), ix.workspace_size(nq, k, ef)
+    assert full > least
+    ref = ix.search(q, k, ef, kernel=1)
+    for size in (least, full):
+        ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+        assert same(ix.search(q, k, ef, workspace=ws), ref)
+    with pytest.raises(B.SqgError):
+        ix.search(q, k, ef, workspace=torch.empty(least - 256, dtype=torch.uint8, device="cuda"))
+    # the fixed scratch: the most queries whose least plan fits it
+    limit = B.lib().sqg_noalloc_scratch_bytes()
+    n = max(m for m in range(100, nq + 1, 50) if ix.workspace_size(m, k, ef, kernel=1) + 32768 <= limit)
+    kt, et = (torch.full((n,), v, dtype=torch.int32, device="cuda") for v in (k, ef))
+    ids, d = torch.empty(n * k, dtype=torch.int32, device="cuda"), torch.empty(n * k, device="cuda")
+    rc = B.lib().sqg_search_noalloc(ix.handle, q.data_ptr(), n, kt.data_ptr(), et.data_ptr(), k, ef, ids.data_ptr(),
+                                    d.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    assert rc == 0 and torch.equal(ids.view(n, k), ref[0][:n]) and torch.equal(d.view(n, k), ref[1][:n])
+
+
+@pytest.mark.parametrize("nq", [1, 3, 64, 700])
+def test_tables_of_a_resident_batch(gpu_tiny, nq):
+    """Batches whose queries are all resident take larger visited tables: the
+    searches of any batch size are the same."""
+    ix, _, q = gpu_tiny
+    qd = torch.from_numpy(np.concatenate([q] * 160)).cuda()  # past the resident warps: the small tables
+    for k, ef in ((10, 64), (100, 160), (64, 400), (10, 1200)):
+        ids, dists, st = ix.search(qd, k, ef, stats=True)
+        assert same(ix.search(qd[:nq], k, ef, stats=True), (ids[:nq], dists[:nq], st[:nq]))
