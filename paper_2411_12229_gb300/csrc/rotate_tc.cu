@@ -595,7 +595,10 @@ cudaError_t launch_quantize_exact(const float *q, const float *rot, const float 
     if (d > kMaxD || d % 32 != 0) return cudaErrorInvalidValue;
     if (nq <= 0) return cudaSuccess;
     const size_t smem = kQxWarps * QxLayout(d).warp;
-    cudaError_t e = cudaFuncSetAttribute(quantize_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the largest d's size whatever d is: the limit is the process's, and calls
+    // of several threads on indexes of different d must not lower it)
+    cudaError_t e = cudaFuncSetAttribute(quantize_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kQxWarps * QxLayout(kMaxD).warp));
     if (e != cudaSuccess) return e;
     quantize_exact_kernel<<<(nq + kQxWarps - 1) / kQxWarps, kQxWarps * 32, smem, s>>>(
         q, rot, qa, nq, d, rotate_tc_err_scale(d), planes, scal, recomputed, plane_major ? 1 : 0, queue);

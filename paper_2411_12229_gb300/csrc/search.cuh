@@ -1018,6 +1018,15 @@ __global__ void __launch_bounds__(128, (LEAN ? 8 : (CH <= 2 ? 5 : 3))) search_ke
 // sqg_workspace_size, or (generous false) the least workspace a search accepts (sqg_api.cu).
 size_t workspace_need(const sqg_index *ix, int nq, int max_k, int max_ef, bool generous);
 
+// Lets a kernel be launched with any dynamic shared memory a block may have
+// (227 KB on sm_103a).  Every call sets the same value: a kernel's limit is one
+// for the whole process, and a thread that set its own size could lower it
+// between another thread's setting and its launch, which was then refused.
+template <class K>
+inline cudaError_t allow_dynamic_smem(K kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+}
+
 // Host-side launch helpers, defined in the instantiation units.
 // Tensor-core rotation and the exact quantization after it (rotate_tc.cu).
 float rotate_tc_err_scale(int d);

@@ -24,8 +24,11 @@
 //     binary search; the merged beam is gathered into the other of two
 //     beam buffers, each output slot finding its source from a 32 NB-bit
 //     mask of the candidates' final positions (no shifting loop);
+//   * with out-degree 32 one or two admitted candidates are inserted into the
+//     registers directly (position by ballots, later entries up by shuffles);
 //   * the k <= 32 RK results live in registers, lane l holding results
-//     l + 32 s (s < RK);
+//     l + 32 s (s < RK); without the stop, more than 32 results are logged
+//     and sorted instead;
 //   * with out-degree 64 (NR = 2) lane l estimates neighbours l and l + 32
 //     and the step's candidates are staged 64 wide.
 //
@@ -330,7 +333,10 @@ __device__ __forceinline__ uint64_t pick(const uint64_t (&b)[NB], int s) {
 // learned early stop fused (the same features, network and decision points
 // as search_kernel's, so the same hops, results and status bits).  RK:
 // result slots per lane (1: k <= 32, 4: k <= 128), lane l holding results
-// l + 32 s.
+// l + 32 s.  What bounds it, measured: the chain of dependent steps of an
+// expansion (475 warp-instructions; a lone warp takes 5.9 cycles for each) and
+// with a full SM the issue slots (2.8 of 4 per cycle); no wait for a block
+// finds it late at any load.
 template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1>
 __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchArgs a) {
     using namespace compact;
@@ -824,7 +830,7 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
 template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1>
 static cudaError_t compact_launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t s, const SearchArgs &a) {
     auto fn = search_compact_kernel<CH, NR, NB, MINB, STOP, RK>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(fn);
     if (e != cudaSuccess) return e;
     fn<<<grid, block, smem, s>>>(a);
     return cudaGetLastError();
@@ -833,7 +839,7 @@ static cudaError_t compact_launch_one(dim3 grid, dim3 block, size_t smem, cudaSt
 template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1>
 static cudaError_t compact_occ_one(int block, size_t smem, int *nb) {
     auto fn = search_compact_kernel<CH, NR, NB, MINB, STOP, RK>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(fn);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, fn, block, smem);
 }

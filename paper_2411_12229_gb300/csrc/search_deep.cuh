@@ -39,7 +39,7 @@
 // ef at every merge.
 //
 // Measured (16,384 candidate searches of d 128 at ef 400, k 64, with the
-// path): 5.29 ms with the general kernel, 2.73 ms here, 1,140 and 700
+// path): 5.29 ms with the general kernel, 2.60 ms here, 1,140 and 700
 // warp-instructions per expansion; bound by issue (2.86 of 4 instructions per
 // cycle, 26 warps per SM).  At d 1536 it is bound by the latency of one
 // expansion (IPC 1.1, 9 warps per SM): the longest queries end the launch.
@@ -511,7 +511,7 @@ __global__ void __launch_bounds__(128, MINB) search_deep_kernel(const SearchArgs
 template <int CH, int NR, int RK, int MINB>
 static cudaError_t deep_launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t s, const SearchArgs &a) {
     auto fn = search_deep_kernel<CH, NR, RK, MINB>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(fn);
     if (e != cudaSuccess) return e;
     fn<<<grid, block, smem, s>>>(a);
     return cudaGetLastError();
@@ -520,7 +520,7 @@ static cudaError_t deep_launch_one(dim3 grid, dim3 block, size_t smem, cudaStrea
 template <int CH, int NR, int RK, int MINB>
 static cudaError_t deep_occ_one(int block, size_t smem, int *nb) {
     auto fn = search_deep_kernel<CH, NR, RK, MINB>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(fn);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, fn, block, smem);
 }

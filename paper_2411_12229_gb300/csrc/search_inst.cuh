@@ -14,7 +14,7 @@ namespace sqg {
 template <int CH, bool LEAN>
 static cudaError_t launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t s, const SearchArgs &a) {
     auto fn = search_kernel<CH, SQG_NB, LEAN>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(fn);
     if (e != cudaSuccess) return e;
     fn<<<grid, block, smem, s>>>(a);
     return cudaGetLastError();
@@ -23,7 +23,7 @@ static cudaError_t launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t s
 template <int CH, bool LEAN>
 static cudaError_t occ_one(int block, size_t smem, int *nb) {
     auto fn = search_kernel<CH, SQG_NB, LEAN>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(fn);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, fn, block, smem);
 }

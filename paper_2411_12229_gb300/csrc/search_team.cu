@@ -7,7 +7,7 @@ namespace sqg {
 template <int CH, int NB, int T>
 static cudaError_t team_launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t s, const SearchArgs &a) {
     auto fn = search_kernel<CH, NB, false, T>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(fn);
     if (e != cudaSuccess) return e;
     fn<<<grid, block, smem, s>>>(a);
     return cudaGetLastError();
@@ -16,7 +16,7 @@ static cudaError_t team_launch_one(dim3 grid, dim3 block, size_t smem, cudaStrea
 template <int CH, int NB, int T>
 static cudaError_t team_occ_one(int block, size_t smem, int *nb) {
     auto fn = search_kernel<CH, NB, false, T>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(fn);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, fn, block, smem);
 }

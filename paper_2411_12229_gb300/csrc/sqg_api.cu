@@ -1130,7 +1130,7 @@ extern "C" int sqg_estimate_block(const sqg_index *ix, const float *queries, int
     a.warp_bytes = (uint32_t)align_up(ix->lay.block_bytes + 16 * (d / 32), 16);
     const int wpb = 2;
     const size_t smem = (size_t)wpb * a.warp_bytes;
-    cudaError_t e = cudaFuncSetAttribute(estimate_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(estimate_block_kernel);
     if (e == cudaSuccess) {
         estimate_block_kernel<<<(nq + wpb - 1) / wpb, wpb * 32, smem, stream>>>(a, v, out_S, out_est, out_key,
                                                                                out_dist_c);

@@ -58,25 +58,59 @@ def test_refused_as_before(gpu_tiny):
                                 B.C.byref(p), None, 0, None, None) == -1
 
 
-def test_threads_share_the_handles_pool(gpu_tiny):
-    ix, q = gpu_tiny
-    qd = torch.from_numpy(q).cuda()
-    ref = ix.search(qd, 10, 64)
+def run_threads(jobs):
+    """Each job in a thread of its own; their exceptions and False results."""
     bad = []
 
-    def work():
-        s = torch.cuda.Stream()
-        with torch.cuda.stream(s):
-            for _ in range(20):
-                ids, dists = ix.search(qd, 10, 64)
-                s.synchronize()
-                if not (torch.equal(ids, ref[0]) and torch.equal(dists, ref[1])):
-                    bad.append(1)
+    def work(job):
+        try:
+            if not job():
+                bad.append("wrong results")
+        except Exception as e:  # noqa: BLE001
+            bad.append(repr(e))
 
     torch.cuda.synchronize()
-    ts = [threading.Thread(target=work) for _ in range(4)]
+    ts = [threading.Thread(target=work, args=(j,)) for j in jobs]
     for t in ts:
         t.start()
     for t in ts:
         t.join()
-    assert not bad
+    return bad
+
+
+def searcher(ix, q, k, ef, reps, **kw):
+    ref = ix.search(q, k, ef, **kw)
+
+    def job():
+        s = torch.cuda.Stream()
+        ok = True
+        with torch.cuda.stream(s):
+            for _ in range(reps):
+                got = ix.search(q, k, ef, **kw)
+                s.synchronize()
+                ok = ok and torch.equal(got[0], ref[0]) and torch.equal(got[1], ref[1])
+        return ok
+
+    return job
+
+
+def test_threads_share_the_handles_pool(gpu_tiny):
+    ix, q = gpu_tiny
+    qd = torch.from_numpy(q).cuda()
+    assert run_threads([searcher(ix, qd, 10, 64, 20) for _ in range(4)]) == []
+
+
+def test_threads_with_different_shapes(gpu_tiny, shaped_index_file):
+    """Batches whose kernels are the same but whose shared memory differs (batch
+    size, ef, visited tables, block size), on two indexes at once: no thread's
+    launch is refused."""
+    from paper_2411_12229_gb300.api import Index
+    ix, q = gpu_tiny
+    q1 = torch.from_numpy(q).cuda()
+    big = q1.repeat(200, 1)
+    p, _, qs = shaped_index_file
+    ix2, q2 = Index(p, 0), torch.from_numpy(qs).cuda()
+    jobs = [searcher(ix, q1, 10, 64, 60), searcher(ix, big, 10, 64, 20), searcher(ix, q1, 10, 50, 60, visited_smem_log2=11),
+            searcher(ix, q1, 10, 400, 40), searcher(ix, q1, 10, 900, 40), searcher(ix, q1, 10, 64, 60, kernel=1),
+            searcher(ix2, q2, 10, 64, 60), searcher(ix2, q2, 10, 300, 40), searcher(ix, q1, 10, 64, 60, warps_per_block=1)]
+    assert run_threads(jobs) == []
