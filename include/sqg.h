@@ -97,7 +97,8 @@ typedef struct {
     void *timing_events[2];  /* optional cudaEvent_t pair recorded on the stream right before
                                 and right after the search kernel; NULL = none */
     int32_t visited_smem_log2; /* log2 of the visited set's shared-memory slots (5..12;
-                                  0 = 9); a search past half of them continues in a
+                                  0 = 9, or up to 11 for a batch whose queries are all
+                                  resident at once); a search past half of them continues in a
                                   full-size table in the workspace */
     int32_t prefetch;        /* 1 (default, 0): the next block is copied into shared
                                 memory during the merge; 2: also L2-prefetch the
@@ -122,9 +123,12 @@ typedef struct {
                                 (one warp per query, d <= 1024, degree 32 or 64, every k[i] <= 32
                                 and ef[i] <= 128 by max_k / max_ef -- for d <= 256 k[i] <= 128
                                 and ef[i] <= 256 --, multiple estimates, no trace, prefetch 1;
-                                with or without the learned stop), else the general one;
+                                with or without the learned stop), else the deep-beam one
+                                (any ef, k <= 128, d <= 2048, multiple estimates, prefetch 1,
+                                no learned stop, no feature trace; also for path traces), else
+                                the general one;
                                 1 = always the general kernel; 2 = the compact kernel or
-                                SQG_ERR_UNSUPPORTED.  Both return identical results. */
+                                SQG_ERR_UNSUPPORTED.  All return identical results. */
     int32_t uniform_k;       /* 0 (default): k[] may differ per query, outputs ragged at the
                                 exclusive prefix sum of k[] (a planning kernel computes it);
                                 > 0: every k[i] is this value, query i's outputs start at
@@ -206,8 +210,9 @@ size_t sqg_workspace_size(const sqg_index *ix, int nq, int max_k, int max_ef);
  *            padded with (SQG_NO_ID, +inf) when fewer vertices were reached.
  *            A query with invalid k or ef contributes max(0, min(k,
  *            SQG_MAX_K)) slots, all padding, and sets SQG_STATUS_BAD_PARAM.
- * Scratch is taken from the stream-ordered allocator on `stream`.  The
- * call synchronizes the stream once to read the batch's largest k and ef.
+ * Scratch is taken from the stream-ordered allocator on `stream` (from the
+ * index's second such call on, from a pool of its own that keeps up to 256
+ * MiB until the index is freed).  The call synchronizes the stream once to read the batch's largest k and ef.
  * SQG_ERR_INVALID_ARG for null pointers or nq < 0 (nq = 0 is a no-op). */
 int sqg_search(const sqg_index *ix, const float *queries, int nq, const int32_t *k, const int32_t *ef,
                uint32_t *out_ids, float *out_dists, sqg_stream_t stream);
