@@ -108,9 +108,10 @@ typedef struct {
                                 default), 2 = the 96-register build (and never the
                                 compact kernel).  Compact kernel: 0 = the build for 8
                                 resident blocks of 4 warps per SM (64 registers) up to
-                                ef 64 and for 7 (72) up to ef 128 with k <= 32; 1 = one
-                                block more (56 / 64 registers); ignored past ef 128 or
-                                k 32 */
+                                ef 64 and for 7 (72) up to ef 128 with k <= 32, or for
+                                batches of at most 8 queries per SM (out-degree 32) a
+                                build for 4; 1 = one block more (56 / 64 registers);
+                                ignored past ef 128 or k 32 */
     int32_t rotation;        /* q' = P^-1 q: 1 = the canonical fp32 order (see
                                 sqg_prepare_queries) on the CUDA cores; 2 = tcgen05 tensor
                                 cores (3xTF32) followed by an exact pass that recomputes in

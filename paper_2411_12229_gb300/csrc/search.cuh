@@ -1053,7 +1053,9 @@ cudaError_t search_occupancy_nb2(int ch, int block, size_t smem, int *blocks_per
 // 4) beam entries (for d <= 256 also k <= 128 and ef <= 256: the big
 // builds below), whole warps, multiple estimates, no trace
 // (lean 1, d <= 256 and out-degree 32: the build for one more resident block
-// of 4 warps per SM: 9 / 8, else 8 / 7)
+// of 4 warps per SM: 9 / 8, else 8 / 7; lean kLeanIdle, same shapes: the build
+// for launches of a few warps per SM)
+constexpr int kLeanIdle = 3;
 cudaError_t launch_search_compact(int ch, int nr, int bnb, int lean, dim3 grid, dim3 block, size_t smem,
                                   cudaStream_t s, const SearchArgs &a);
 cudaError_t search_occupancy_compact(int ch, int nr, int bnb, int lean, int block, size_t smem, int *blocks_per_sm);

@@ -121,37 +121,75 @@ __device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
 // for 2 LOP3 each.  Exact partial, S and butterfly at d 960, out-degree 64,
 // cycles per expansion, word by word / here: 4,160 / 2,780 for a lone warp,
 // 6,250 / 4,600 with 12 warps per SM.  A second adder level gains nothing
-// (4,800: the ALU is then the limit).  For d <= 256, where other ALU work
-// dominates a full SM, adders cost more than they save (10k queries of d 128,
-// ef 40: 262 us word by word, 273 with adders).
-template <int CH, int NR>
+// (4,800: the ALU is then the limit).  For d <= 256 other ALU work dominates a
+// full SM, and adders cost more than they save (10k queries of d 128, ef 40:
+// 262 us word by word, 273 with adders); where issue slots are free the chain
+// they shorten counts (ADD: exact partial, S and butterfly of a lone warp 595
+// -> 289 cycles).
+template <int CH, int NR, bool ADD>
 __device__ __forceinline__ void exact_and_S(const float4 (&qv)[CH], const unsigned char *blk, uint32_t off_codes,
-                                            const uint32_t *planes, uint32_t nch, uint32_t nw, int lane,
-                                            float (&acc)[1], int (&S)[NR]) {
+                                            const uint32_t *planes, uint32_t nch, uint32_t nw, int lane, float (&acc)[1],
+                                            int (&S)[NR]) {
     constexpr uint32_t R = 32 * NR;
     const uint32_t *codes = reinterpret_cast<const uint32_t *>(blk + off_codes) + lane;
     const uint4 *pl = reinterpret_cast<const uint4 *>(planes);
     if constexpr (CH <= 2) {
         exact_partial<CH, 32>(reinterpret_cast<const float4(&)[1][CH]>(qv), reinterpret_cast<const float *>(blk), nch,
                               Team<32>(lane), acc);
-        int s0[NR], s1[NR], s2[NR], s3[NR];
+        if constexpr (NR == 1 && ADD) {
+            // groups of four words, absent words zero; within a group the carries
+            // of plane b join plane b + 1's words: 9 POPCs for 16
+            S[0] = 0;
 #pragma unroll
-        for (int n = 0; n < NR; ++n) s0[n] = s1[n] = s2[n] = s3[n] = 0;
+            for (uint32_t g = 0; g < 4 * CH; g += 4) {
+                if (g > 0 && g >= nw) break;
+                uint32_t c[4], p[4][4];  // [plane][word]
 #pragma unroll
-        for (uint32_t w = 0; w < 4 * CH; ++w)
-            if (w < nw) {
-                const uint4 p = pl[w];
-#pragma unroll
-                for (int n = 0; n < NR; ++n) {
-                    const uint32_t c = codes[w * R + 32 * n];
-                    s0[n] += __popc(c & p.x);
-                    s1[n] += __popc(c & p.y);
-                    s2[n] += __popc(c & p.z);
-                    s3[n] += __popc(c & p.w);
+                for (uint32_t w = 0; w < 4; ++w) {
+                    const bool in = g + w < nw;
+                    const uint4 v = in ? pl[g + w] : make_uint4(0u, 0u, 0u, 0u);
+                    p[0][w] = v.x;
+                    p[1][w] = v.y;
+                    p[2][w] = v.z;
+                    p[3][w] = v.w;
+                    c[w] = in ? codes[(g + w) * R] : 0u;
                 }
-            }
+                uint32_t s0[4], c0[4], a3[4], u[4], t[4];
 #pragma unroll
-        for (int n = 0; n < NR; ++n) S[n] = s0[n] + 2 * s1[n] + 4 * s2[n] + 8 * s3[n];
+                for (int b = 0; b < 4; ++b) {
+                    const uint32_t x = c[0] & p[b][0], y = c[1] & p[b][1], z = c[2] & p[b][2];
+                    s0[b] = xor3(x, y, z);  // weight 2^b
+                    c0[b] = maj3(x, y, z);  // weight 2^(b + 1)
+                    a3[b] = c[3] & p[b][3];
+                }
+#pragma unroll
+                for (int b = 1; b < 4; ++b) {
+                    t[b] = xor3(c0[b - 1], s0[b], a3[b]);
+                    u[b] = maj3(c0[b - 1], s0[b], a3[b]);
+                }
+                S[0] += __popc(s0[0]) + __popc(a3[0]) + 2 * __popc(t[1]) + 4 * (__popc(t[2]) + __popc(u[1])) +
+                        8 * (__popc(t[3]) + __popc(u[2])) + 16 * (__popc(c0[3]) + __popc(u[3]));
+            }
+        } else {
+            int s0[NR], s1[NR], s2[NR], s3[NR];
+    #pragma unroll
+            for (int n = 0; n < NR; ++n) s0[n] = s1[n] = s2[n] = s3[n] = 0;
+    #pragma unroll
+            for (uint32_t w = 0; w < 4 * CH; ++w)
+                if (w < nw) {
+                    const uint4 p = pl[w];
+    #pragma unroll
+                    for (int n = 0; n < NR; ++n) {
+                        const uint32_t c = codes[w * R + 32 * n];
+                        s0[n] += __popc(c & p.x);
+                        s1[n] += __popc(c & p.y);
+                        s2[n] += __popc(c & p.z);
+                        s3[n] += __popc(c & p.w);
+                    }
+                }
+    #pragma unroll
+            for (int n = 0; n < NR; ++n) S[n] = s0[n] + 2 * s1[n] + 4 * s2[n] + 8 * s3[n];
+        }
     } else {
         // chunk t: the lane's t-th float4 of the raw vector and words 4 t .. 4
         // t + 3; `one` carries each plane's sum of weight 1 from word to word
@@ -337,7 +375,7 @@ __device__ __forceinline__ uint64_t pick(const uint64_t (&b)[NB], int s) {
 // expansion (475 warp-instructions; a lone warp takes 5.9 cycles for each) and
 // with a full SM the issue slots (2.8 of 4 per cycle); no wait for a block
 // finds it late at any load.
-template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1>
+template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1, bool ADD = false>
 __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchArgs a) {
     using namespace compact;
     constexpr bool kLog = RK > 1 && !STOP;  // (the stop's features need the results in order)
@@ -466,7 +504,7 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
             int S[NR];
 #pragma unroll
             for (int t = 0; t < NR; ++t) cid[t] = reinterpret_cast<const uint32_t *>(blk + a.off_ids)[lane + 32 * t];
-            exact_and_S<CH, NR>(qv, blk, a.off_codes, planes, nch, d / 32, lane, dacc, S);
+            exact_and_S<CH, NR, ADD>(qv, blk, a.off_codes, planes, nch, d / 32, lane, dacc, S);
             EstPart part[NR];
             uint32_t hv[NR];  // each neighbour's first visited-set slot
 #pragma unroll
@@ -827,18 +865,18 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
     }
 }
 
-template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1>
+template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1, bool ADD = false>
 static cudaError_t compact_launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t s, const SearchArgs &a) {
-    auto fn = search_compact_kernel<CH, NR, NB, MINB, STOP, RK>;
+    auto fn = search_compact_kernel<CH, NR, NB, MINB, STOP, RK, ADD>;
     cudaError_t e = allow_dynamic_smem(fn);
     if (e != cudaSuccess) return e;
     fn<<<grid, block, smem, s>>>(a);
     return cudaGetLastError();
 }
 
-template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1>
+template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1, bool ADD = false>
 static cudaError_t compact_occ_one(int block, size_t smem, int *nb) {
-    auto fn = search_compact_kernel<CH, NR, NB, MINB, STOP, RK>;
+    auto fn = search_compact_kernel<CH, NR, NB, MINB, STOP, RK, ADD>;
     cudaError_t e = allow_dynamic_smem(fn);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, fn, block, smem);

@@ -2,7 +2,10 @@
 // for d <= 256 with beams of 129-256 entries (NB = 8 slots per lane) or
 // with 33-128 results (RK = 4 slots per lane), plain and with the learned
 // stop fused.  Resident blocks of 4 warps per SM: the most at which the
-// build does not spill (80 registers for 6 blocks, 96 for 5).
+// build does not spill (80 registers for 6 blocks, 96 for 5).  With four
+// result slots the estimates use adders (10,000 queries of d 128, k 100, ef
+// 200: 1,116 -> 1,098 us; 2,001: 401 -> 380), with one they do not (k 10, ef
+// 160: 827 against 864).
 #include "search_compact.cuh"
 
 namespace sqg {
@@ -32,14 +35,14 @@ namespace sqg {
 
 cudaError_t launch_search_compact_big(int ch, int nr, int bnb, int rk, bool stop, dim3 grid, dim3 block, size_t smem,
                                       cudaStream_t s, const SearchArgs &a) {
-#define CALL(C, R, N, M, S, K) compact_launch_one<C, R, N, M, S, K>(grid, block, smem, s, a)
+#define CALL(C, R, N, M, S, K) compact_launch_one<C, R, N, M, S, K, !S && K == 4>(grid, block, smem, s, a)
     SQG_COMPACT_BIG_SWITCH(CALL)
 #undef CALL
 }
 
 cudaError_t search_occupancy_compact_big(int ch, int nr, int bnb, int rk, bool stop, int block, size_t smem,
                                          int *blocks_per_sm) {
-#define CALL(C, R, N, M, S, K) compact_occ_one<C, R, N, M, S, K>(block, smem, blocks_per_sm)
+#define CALL(C, R, N, M, S, K) compact_occ_one<C, R, N, M, S, K, !S && K == 4>(block, smem, blocks_per_sm)
     SQG_COMPACT_BIG_SWITCH(CALL)
 #undef CALL
 }

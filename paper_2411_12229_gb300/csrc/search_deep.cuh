@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(128, MINB) search_deep_kernel(const SearchArgs
             int S[NR];
 #pragma unroll
             for (int t = 0; t < NR; ++t) cid[t] = reinterpret_cast<const uint32_t *>(blk + a.off_ids)[lane + 32 * t];
-            exact_and_S<CH, NR>(qv, blk, a.off_codes, planes, nch, d / 32, lane, dacc, S);
+            exact_and_S<CH, NR, false>(qv, blk, a.off_codes, planes, nch, d / 32, lane, dacc, S);
             EstPart part[NR];
             uint32_t hv[NR];  // each neighbour's first visited-set slot
 #pragma unroll

@@ -404,6 +404,7 @@ struct LaunchPlan {
     int ch, nb, team, warps, grid;
     bool compact;  // the compact kernel (search_compact.cu)
     bool deep;     // the deep-beam kernel (search_deep.cu)
+    int lean;      // the compact kernel's build (params.lean, or kLeanIdle)
     int cbnb;      // its beam slots per lane: 2 (ef <= 64), 4 (ef <= 128) or 8 (ef <= 256, d <= 256)
     int crk;       // its result slots per lane: 1 (k <= 32) or 4 (k <= 128, d <= 256)
     size_t smem;
@@ -444,6 +445,10 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
               traced != kTraceFeatures && p.prefetch != 2 && p.lean != 2;
     pl.cbnb = max_ef <= 64 ? 2 : max_ef <= 128 ? 4 : 8;
     pl.crk = max_k <= 32 ? 1 : 4;
+    // Up to eight queries per SM leave most issue slots free: a build with twice
+    // the registers and shorter chains (one query of d 128: 73 -> 65 us, 200: 92
+    // -> 79, 1,200: 133 -> 114, at ef 100 186 -> 170).
+    pl.lean = p.lean == 0 && pl.ch <= 2 && pl.nb == 1 && nq <= 8 * ix->num_sms ? kLeanIdle : p.lean;
     const bool big = pl.compact && (pl.cbnb == 8 || pl.crk == 4);  // search_compact_big.cu
     if (pl.compact || pl.deep) {
     } else if (pl.team < 32) {
@@ -512,7 +517,7 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
         return big ? search_occupancy_compact_big(pl.ch, pl.nb, pl.cbnb, pl.crk, p.stop_mlp != nullptr, w * 32, sm,
                                                   blocks)
              : pl.compact && p.stop_mlp ? search_occupancy_compact_stop(pl.ch, pl.nb, pl.cbnb, w * 32, sm, blocks)
-             : pl.compact     ? search_occupancy_compact(pl.ch, pl.nb, pl.cbnb, p.lean, w * 32, sm, blocks)
+             : pl.compact     ? search_occupancy_compact(pl.ch, pl.nb, pl.cbnb, pl.lean, w * 32, sm, blocks)
              : pl.deep        ? search_occupancy_deep(pl.ch, pl.nb, pl.crk, w * 32, sm, blocks)
              : pl.team < 32 ? search_occupancy_team(pl.ch, pl.nb, pl.team, w * 32, sm, blocks)
              : pl.nb == 1   ? search_occupancy_nb1(pl.ch, w * 32, sm, blocks)
@@ -986,7 +991,7 @@ static int search_impl(const sqg_index *ix, const float *queries, int nq, const 
             : pl.compact && p.stop_mlp
                 ? launch_search_compact_stop(pl.ch, pl.nb, pl.cbnb, dim3(pl.grid), dim3(pl.warps * 32), pl.smem,
                                              stream, a)
-            : pl.compact ? launch_search_compact(pl.ch, pl.nb, pl.cbnb, p.lean, dim3(pl.grid), dim3(pl.warps * 32),
+            : pl.compact ? launch_search_compact(pl.ch, pl.nb, pl.cbnb, pl.lean, dim3(pl.grid), dim3(pl.warps * 32),
                                                  pl.smem, stream, a)
             : pl.deep    ? launch_search_deep(pl.ch, pl.nb, pl.crk, dim3(pl.grid), dim3(pl.warps * 32), pl.smem,
                                               stream, a)
