@@ -371,7 +371,8 @@ __device__ __forceinline__ uint64_t pick(const uint64_t (&b)[NB], int s) {
 // learned early stop fused (the same features, network and decision points
 // as search_kernel's, so the same hops, results and status bits).  RK:
 // result slots per lane (1: k <= 32, 4: k <= 128), lane l holding results
-// l + 32 s.  What bounds it, measured: the chain of dependent steps of an
+// l + 32 s.  ADD: full adders in the estimates (exact_and_S).  What bounds
+// it, measured: the chain of dependent steps of an
 // expansion (475 warp-instructions; a lone warp takes 5.9 cycles for each) and
 // with a full SM the issue slots (2.8 of 4 per cycle); no wait for a block
 // finds it late at any load.
