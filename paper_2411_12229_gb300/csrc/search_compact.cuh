@@ -372,10 +372,10 @@ __device__ __forceinline__ uint64_t pick(const uint64_t (&b)[NB], int s) {
 // as search_kernel's, so the same hops, results and status bits).  RK:
 // result slots per lane (1: k <= 32, 4: k <= 128), lane l holding results
 // l + 32 s.  ADD: full adders in the estimates (exact_and_S).  What bounds
-// it, measured: the chain of dependent steps of an
-// expansion (475 warp-instructions; a lone warp takes 5.9 cycles for each) and
-// with a full SM the issue slots (2.8 of 4 per cycle); no wait for a block
-// finds it late at any load.
+// it, measured: the chain of dependent steps of an expansion (without ADD 475
+// warp-instructions; a lone warp takes 5.9 cycles for each) and with a full SM
+// the issue slots (2.8 of 4 per cycle); no wait for a block finds it late at
+// any load.
 template <int CH, int NR, int NB, int MINB, bool STOP = false, int RK = 1, bool ADD = false>
 __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchArgs a) {
     using namespace compact;
