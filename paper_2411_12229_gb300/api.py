@@ -21,6 +21,34 @@ def _stream_ptr(stream) -> int:
     return int(s.cuda_stream)
 
 
+def _launch_stream(stream, device):
+    """A caller's stream (any object with a ``cuda_stream``) as a torch stream;
+    None if it is torch's current stream or not given."""
+    if stream is None or int(stream.cuda_stream) == int(torch.cuda.current_stream(device).cuda_stream):
+        return None
+    if isinstance(stream, torch.cuda.Stream):
+        return stream
+    return torch.cuda.ExternalStream(int(stream.cuda_stream), device=device)
+
+
+def _order_after_current(side, device, *tensors) -> None:
+    """Before a launch on `side` (of _launch_stream): the launch comes after
+    what torch's current stream holds -- the padding, copies and fills of the
+    call itself and whatever produced the caller's tensors -- and the memory of
+    the tensors (None: absent) is not handed out again before it is done.
+    Where one of the two streams is being captured and the other is not, the
+    order is the caller's."""
+    if side is None:
+        return
+    with torch.cuda.stream(side):
+        captured = torch.cuda.is_current_stream_capturing()
+    if captured == torch.cuda.is_current_stream_capturing():
+        side.wait_stream(torch.cuda.current_stream(device))
+    for t in tensors:
+        if t is not None and t.is_cuda:
+            t.record_stream(side)
+
+
 def _scalar(x) -> int | None:
     """x as an int32 value if it is one number, else None."""
     if isinstance(x, torch.Tensor) or np.ndim(x) != 0:
@@ -28,13 +56,13 @@ def _scalar(x) -> int | None:
     return int(np.asarray(x, dtype=np.int32))
 
 
-def _i32(x, nq: int, device, stream=None) -> torch.Tensor:
+def _i32(x, nq: int, device, side=None) -> torch.Tensor:
     """nq int32 values on the device: a tensor or array of them, or one number
     for all (filled on the stream that will read it: a host copy of the array
     would wait for everything the stream still has to do)."""
     one = _scalar(x)
     if one is not None:
-        with torch.cuda.stream(stream):
+        with torch.cuda.stream(side):
             return torch.full((nq,), one, dtype=torch.int32, device=device)
     if isinstance(x, torch.Tensor):
         t = x.to(device=device, dtype=torch.int32).contiguous()
@@ -124,7 +152,12 @@ class Index:
         (or (nq, uniform_k) with that keyword), else flat ragged arrays
         (query i at offset sum_{j<i} k[j]).  Padding
         is id -1 with distance +inf.  With stats=True also returns an
-        (nq, 2) int32 tensor of (hops, status bits)."""
+        (nq, 2) int32 tensor of (hops, status bits).
+
+        On a `stream` other than torch's current one the search starts after
+        what the current stream holds at the call, so tensors made there need
+        no order of the caller's; `out`, `workspace` and a `stop_mlp` are the
+        caller's to keep until the search is done."""
         queries = self.fit_queries(queries)
         if queries.dtype != torch.float32 or not queries.is_cuda or queries.dim() != 2 or queries.shape[1] != self.d:
             raise ValueError(f"queries must be a CUDA float32 tensor of shape (nq, {self.d})")
@@ -143,8 +176,9 @@ class Index:
         # one k and one ef: passed by value, no arrays (ef < 1 or another
         # uniform_k keeps the arrays and the checks made on them)
         by_value = uniform and ef1 is not None and ef1 >= 1 and 1 <= k1 <= B.MAX_K and p.uniform_k == k1
+        side, kt, et = _launch_stream(stream, dev), None, None
         if not by_value:
-            kt, et = _i32(k, nq, dev, stream), _i32(ef, nq, dev, stream)
+            kt, et = _i32(k, nq, dev, side), _i32(ef, nq, dev, side)
         if out is None:  # (with `out` given nothing here waits on the device)
             total = uk * nq if uk else int(k) * nq if uniform else int(kt.clamp(0, B.MAX_K).sum().item())
             ids = torch.empty(total, dtype=torch.int32, device=dev)
@@ -155,6 +189,8 @@ class Index:
         ws_ptr, ws_bytes = (workspace.data_ptr(), workspace.numel() * workspace.element_size()) \
             if workspace is not None else (None, 0)
         st_ptr = st.data_ptr() if st is not None else None
+        made = (ids, dists) if out is None else ()
+        _order_after_current(side, dev, queries, kt, et, st, *made)
         if by_value:
             rc = B.lib().sqg_search_uniform(self._h, queries.data_ptr(), nq, k1, ef1, ids.data_ptr(),
                                             dists.data_ptr(), C.byref(p), ws_ptr, ws_bytes, st_ptr,
@@ -181,9 +217,10 @@ class Index:
         gt) at every evaluation point, and/or the expansion order.  Returns
         ids, dists, stats, feats (nq, cap, 16), hits (nq, cap), counts (nq,)
         and, with path_cap > 0, path (nq, path_cap; -1 past the last hop)."""
-        queries = self.fit_queries(queries)
+        queries = self.fit_queries(queries).contiguous()
         nq, dev = queries.shape[0], queries.device
-        kt, et = _i32(k, nq, dev, stream), _i32(ef, nq, dev, stream)
+        side = _launch_stream(stream, dev)
+        kt, et = _i32(k, nq, dev, side), _i32(ef, nq, dev, side)
         ids = torch.empty(nq * k, dtype=torch.int32, device=dev)
         dists = torch.empty(nq * k, dtype=torch.float32, device=dev)
         st = torch.empty((nq, 2), dtype=torch.int32, device=dev)
@@ -196,7 +233,8 @@ class Index:
         p = self.params(max_k=k, max_ef=ef, **{"uniform_k": k, **kw})  # rows of k: no planning kernel
         gtp, gtk = (gt.data_ptr(), gt.shape[1]) if gt is not None else (None, 0)
         ptr = lambda t: t.data_ptr() if t is not None else None  # noqa: E731
-        rc = B.lib().sqg_search_trace(self._h, queries.contiguous().data_ptr(), nq, kt.data_ptr(), et.data_ptr(),
+        _order_after_current(side, dev, queries, kt, et, gt, ids, dists, st, feats, hits, cnt, path)
+        rc = B.lib().sqg_search_trace(self._h, queries.data_ptr(), nq, kt.data_ptr(), et.data_ptr(),
                                       ids.data_ptr(), dists.data_ptr(), C.byref(p), st.data_ptr(), gtp, gtk,
                                       ptr(feats), ptr(hits), ptr(cnt), trace_cap, ptr(path), path_cap,
                                       _stream_ptr(stream))
