@@ -163,14 +163,16 @@ __global__ void __launch_bounds__(kThreads) mlp_grad_kernel(const float *__restr
 #pragma unroll
                 for (int o = 8; o >= 1; o >>= 1) p += __shfl_xor_sync(0xFFFFFFFFu, p, o);  // the 16 threads of a sample
                 const float z = p + b3, yy = s.y[r], ww = s.w[r];
-                const float dz = ww * (1.0f / (1.0f + expf(-z)) - yy);  // 0 for an absent sample (ww = 0)
-                if (tx == 0) {
+                // (an absent sample takes no part: its z may overflow where no real one does)
+                const bool here = r < rows;
+                const float dz = here ? ww * (1.0f / (1.0f + expf(-z)) - yy) : 0.f;
+                if (tx == 0 && here) {
                     lsum += ww * (softplus(z) - yy * z);
                     gb3 += dz;
                 }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const bool on = a[i][j] > 0.f;
+                    const bool on = here && a[i][j] > 0.f;
                     const float d2 = on ? dz * w3[j] : 0.f;
                     gW3[j] = fmaf(dz, on ? a[i][j] : 0.f, gW3[j]);
                     gb2[j] += d2;
