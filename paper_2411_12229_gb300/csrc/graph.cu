@@ -552,14 +552,19 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
     }
     int rc = SQG_OK;
     {
-        DevArena A;
-        const size_t o_data = A.add(sizeof(float) * n * d), o_cand = A.add(sizeof(uint32_t) * n * L);
+        // What is not needed at the same time shares memory: the rows, and the
+        // reverse lists where they fit behind them, take the candidate ids'
+        // place once the pruning has read those; the reverse counts, the kept
+        // edges' counts and the flood's levels follow one another.  The reverse
+        // lists are allocated at their real length, about a third of n R'.
+        DevArena A, V;
+        const size_t cand_bytes = sizeof(uint32_t) * n * L;
+        const size_t rows_bytes = (sizeof(uint32_t) * n * R + 255) / 256 * 256;
+        const size_t o_data = A.add(sizeof(float) * n * d), o_cand = A.add(std::max(cand_bytes, rows_bytes));
         const size_t o_own = A.add(sizeof(u64) * n * L), o_cnt = A.add(sizeof(uint32_t) * n);
         const size_t o_k1 = A.add(sizeof(u64) * n * Rr), o_n1 = A.add(sizeof(uint32_t) * n);
-        const size_t o_rcnt = A.add(sizeof(uint32_t) * n), o_roff = A.add(sizeof(uint64_t) * (n + 1));
-        const size_t o_rev = A.add(sizeof(u64) * n * Rr), o_k2 = A.add(sizeof(u64) * n * Rr);
+        const size_t o_roff = A.add(sizeof(uint64_t) * (n + 1)), o_k2 = A.add(sizeof(u64) * n * Rr);
         const size_t o_n2 = A.add(sizeof(uint32_t) * n), o_flag = A.add(sizeof(uint32_t) * n);
-        const size_t o_adj = A.add(sizeof(uint32_t) * n * R), o_level = A.add(sizeof(uint32_t) * n);
         constexpr int kBatch = 8;  // flood levels between looks at the result
         const size_t o_ctr = A.add(sizeof(u64) * kCounters), o_grew = A.add(sizeof(uint32_t) * kBatch);
         if (!A.commit()) {
@@ -567,9 +572,10 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
             rc = SQG_ERR_OOM;
         }
         float *d_data = A.at<float>(o_data);
-        uint32_t *c_cnt = A.at<uint32_t>(o_cnt), *n1 = A.at<uint32_t>(o_n1), *rcnt = A.at<uint32_t>(o_rcnt);
-        uint32_t *n2 = A.at<uint32_t>(o_n2), *flag = A.at<uint32_t>(o_flag), *d_adj = A.at<uint32_t>(o_adj);
-        u64 *c_own = A.at<u64>(o_own), *k1 = A.at<u64>(o_k1), *k2 = A.at<u64>(o_k2), *d_rev = A.at<u64>(o_rev);
+        uint32_t *c_cnt = A.at<uint32_t>(o_cnt), *n1 = A.at<uint32_t>(o_n1), *flag = A.at<uint32_t>(o_flag);
+        uint32_t *d_cand = A.at<uint32_t>(o_cand), *d_adj = d_cand;
+        uint32_t *n2 = A.at<uint32_t>(o_n2), *rcnt = n2, *level = n2;
+        u64 *c_own = A.at<u64>(o_own), *k1 = A.at<u64>(o_k1), *k2 = A.at<u64>(o_k2), *d_rev = nullptr;
         uint64_t *d_roff = A.at<uint64_t>(o_roff);
         u64 *ctr = A.at<u64>(o_ctr), h_ctr[kCounters] = {};
         int sms = 0;
@@ -586,14 +592,29 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
             ok(cudaMemcpy(d_data, data, sizeof(float) * n * d, cudaMemcpyHostToDevice))) {
             finite_kernel<<<sms * 4, 256>>>(d_data, n * d, ctr);
             ok(cudaGetLastError());
-            ok(cudaMemcpy(A.at<uint32_t>(o_cand), cand, sizeof(uint32_t) * n * L, cudaMemcpyHostToDevice));
+            ok(cudaMemcpy(d_cand, cand, cand_bytes, cudaMemcpyHostToDevice));
             ok(cudaMemcpy(h_ctr, ctr, sizeof(h_ctr), cudaMemcpyDeviceToHost));
             if (rc == SQG_OK && h_ctr[kBadValues]) rc = SQG_ERR_INVALID_ARG;
         }
-        if (rc == SQG_OK) {  // (1)-(3)
-            adjust_prune_kernel<<<grid, kWarps * 32>>>(d_data, n, d, A.at<uint32_t>(o_cand), L, Rr, c_own, c_cnt, k1, n1,
-                                                       rcnt, ctr);
+        if (rc == SQG_OK) {  // (1), and the reverse lists' lengths
+            adjust_prune_kernel<<<grid, kWarps * 32>>>(d_data, n, d, d_cand, L, Rr, c_own, c_cnt, k1, n1, rcnt, ctr);
             reverse_offsets_kernel<<<1, kScanThreads>>>(rcnt, n, d_roff);
+            ok(cudaGetLastError());
+            ok(cudaMemcpy(h_ctr, ctr, sizeof(h_ctr), cudaMemcpyDeviceToHost));  // (the pruning is done)
+            const size_t rev_bytes = sizeof(u64) * h_ctr[kSumKept];
+            if (rows_bytes + rev_bytes <= cand_bytes) {
+                d_rev = A.at<u64>(o_cand + rows_bytes);
+            } else {
+                V.add(rev_bytes);
+                if (V.commit()) {
+                    d_rev = V.at<u64>(0);
+                } else {
+                    cudaGetLastError();
+                    if (rc == SQG_OK) rc = SQG_ERR_OOM;
+                }
+            }
+        }
+        if (rc == SQG_OK) {  // (2)-(3)
             reverse_fill_kernel<<<warp_blocks, 256>>>(k1, n1, n, Rr, d_roff, rcnt, d_rev);
             adjust_refine_kernel<<<grid, kWarps * 32>>>(d_data, n, d, L, Rr, c_own, c_cnt, k1, n1, d_rev, d_roff,
                                                         regular ? 1 : 0, R, k2, n2, flag, d_adj, ctr);
@@ -646,7 +667,7 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
             bool current = !host_rows && !fill_rows;  // d_adj holds them
             const uint64_t repairs = sqg_graph::repair_reachability(
                 n, cand, L, R, entry, out_adj, [&](std::vector<uint8_t> &seen) {
-                    uint32_t *level = A.at<uint32_t>(o_level), *grew = A.at<uint32_t>(o_grew);
+                    uint32_t *grew = A.at<uint32_t>(o_grew);
                     const uint32_t zero = 0;
                     if (!current) ok(cudaMemcpy(d_adj, out_adj, sizeof(uint32_t) * n * R, cudaMemcpyHostToDevice));
                     current = false;  // the repair may change rows before it asks again
