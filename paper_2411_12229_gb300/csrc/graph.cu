@@ -664,9 +664,22 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
                 }, 1);
         }
         if (rc == SQG_OK) {  // (5) reachability, flooded on the device from out_adj's current rows
+            // A level is one launch that looks at every vertex, whatever it reaches:
+            // 5.7 us with its share of the looks at the result (20,000 to 200,000
+            // vertices; 6.6 at a million), while the host's flood looks at every
+            // edge once, 40 to 180 ns per vertex of 32 edges.  A graph of very many
+            // levels is the host's: n / 128 of them take 45 ns per vertex, so the
+            // change costs at most about what the host takes.  A chain of 200,000
+            // vertices: 15 ms for the call, 1,170 with a launch for each level.
+            const uint64_t most = std::max<uint64_t>(64, n / 128);
+            bool deep = false;
             bool current = !host_rows && !fill_rows;  // d_adj holds them
             const uint64_t repairs = sqg_graph::repair_reachability(
                 n, cand, L, R, entry, out_adj, [&](std::vector<uint8_t> &seen) {
+                    if (deep) {
+                        seen = sqg_graph::reachable_host(n, R, entry, out_adj);
+                        return true;
+                    }
                     uint32_t *grew = A.at<uint32_t>(o_grew);
                     const uint32_t zero = 0;
                     if (!current) ok(cudaMemcpy(d_adj, out_adj, sizeof(uint32_t) * n * R, cudaMemcpyHostToDevice));
@@ -681,6 +694,11 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
                         ok(cudaGetLastError());
                         ok(cudaMemcpy(h_grew, grew, sizeof(h_grew), cudaMemcpyDeviceToHost));
                         if (!h_grew[kBatch - 1]) break;
+                        deep = at + kBatch >= most;
+                        if (deep) {
+                            seen = sqg_graph::reachable_host(n, R, entry, out_adj);
+                            return rc == SQG_OK;
+                        }
                     }
                     std::vector<uint32_t> h_level(n);
                     if (!ok(cudaMemcpy(h_level.data(), level, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost))) return false;
