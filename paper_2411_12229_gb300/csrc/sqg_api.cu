@@ -8,9 +8,11 @@
 #include <atomic>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "../../include/sqg.h"
@@ -44,6 +46,10 @@ struct sqg_index {
     // and thread safety are the stream-ordered allocator's own.
     cudaMemPool_t pool;
     mutable std::atomic<bool> scratch_taken{false};
+    // What the driver answered to a plan's questions for a build's resident
+    // blocks per SM: (build, block size, shared memory) << 8 | blocks + 1 in one
+    // word each, so threads need no lock; a new answer takes an old one's place.
+    mutable std::atomic<uint64_t> resident[256] = {};
 };
 
 namespace {
@@ -509,19 +515,34 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
     const size_t cta = 0;  // the stop network's weights are read from the workspace (L1-cached)
     size_t warp_bytes = 0;
     int warps = 0, per_sm = 0;
-    // one slot of warp_bytes per query in flight: V per warp
+    // one slot of warp_bytes per query in flight: V per warp.  The driver is
+    // asked once per build and size (a search asks for three block sizes and up
+    // to three table sizes: 7 us of a call's host time when each was asked anew)
     auto occupancy = [&](int w, int *blocks) -> cudaError_t {
         const size_t sm = cta + (size_t)w * V * warp_bytes;
         *blocks = 0;
         if (sm > ix->smem_optin) return cudaSuccess;
-        return big ? search_occupancy_compact_big(pl.ch, pl.nb, pl.cbnb, pl.crk, p.stop_mlp != nullptr, w * 32, sm,
-                                                  blocks)
-             : pl.compact && p.stop_mlp ? search_occupancy_compact_stop(pl.ch, pl.nb, pl.cbnb, w * 32, sm, blocks)
-             : pl.compact     ? search_occupancy_compact(pl.ch, pl.nb, pl.cbnb, pl.lean, w * 32, sm, blocks)
-             : pl.deep        ? search_occupancy_deep(pl.ch, pl.nb, pl.crk, w * 32, sm, blocks)
-             : pl.team < 32 ? search_occupancy_team(pl.ch, pl.nb, pl.team, w * 32, sm, blocks)
-             : pl.nb == 1   ? search_occupancy_nb1(pl.ch, w * 32, sm, blocks)
-                            : search_occupancy_nb2(pl.ch, w * 32, sm, blocks);
+        uint64_t key = 0;
+        const std::pair<int, unsigned> fields[] = {  // each field's value and width
+            {(int)sm, 18u}, {w, 3u}, {std::abs(pl.ch), 5u}, {pl.ch < 0, 1u}, {pl.nb, 2u}, {pl.cbnb, 4u}, {pl.crk, 3u},
+            {pl.lean, 2u}, {pl.team, 6u}, {pl.compact, 1u}, {pl.deep, 1u}, {p.stop_mlp != nullptr, 1u}};
+        for (const auto &f : fields) key = key << f.second | (uint64_t)f.first;
+        std::atomic<uint64_t> &slot = ix->resident[(key * 0x9E3779B97F4A7C15ull) >> 56];
+        const uint64_t known = slot.load(std::memory_order_relaxed);
+        if (known >> 8 == key && (known & 255u) != 0) {
+            *blocks = (int)(known & 255u) - 1;
+            return cudaSuccess;
+        }
+        const cudaError_t e =
+            big ? search_occupancy_compact_big(pl.ch, pl.nb, pl.cbnb, pl.crk, p.stop_mlp != nullptr, w * 32, sm, blocks)
+            : pl.compact && p.stop_mlp ? search_occupancy_compact_stop(pl.ch, pl.nb, pl.cbnb, w * 32, sm, blocks)
+            : pl.compact     ? search_occupancy_compact(pl.ch, pl.nb, pl.cbnb, pl.lean, w * 32, sm, blocks)
+            : pl.deep        ? search_occupancy_deep(pl.ch, pl.nb, pl.crk, w * 32, sm, blocks)
+            : pl.team < 32 ? search_occupancy_team(pl.ch, pl.nb, pl.team, w * 32, sm, blocks)
+            : pl.nb == 1   ? search_occupancy_nb1(pl.ch, w * 32, sm, blocks)
+                           : search_occupancy_nb2(pl.ch, w * 32, sm, blocks);
+        if (e == cudaSuccess) slot.store(key << 8 | (uint64_t)(*blocks + 1), std::memory_order_relaxed);
+        return e;
     };
     auto residency = [&](uint32_t slots_log2) -> int {
         a.shash_bits = std::min<uint32_t>(bits, slots_log2);
