@@ -97,9 +97,10 @@ typedef struct {
     void *timing_events[2];  /* optional cudaEvent_t pair recorded on the stream right before
                                 and right after the search kernel; NULL = none */
     int32_t visited_smem_log2; /* log2 of the visited set's shared-memory slots (5..12;
-                                  0 = 9, or up to 11 for a batch whose queries are all
-                                  resident at once); a search past half of them continues in a
-                                  full-size table in the workspace */
+                                  0 = 9, or 10 or 11 for a batch whose queries are all
+                                  resident at once, as far as few or no resident warps are
+                                  given up for it); a search past half of them continues in
+                                  a full-size table in the workspace */
     int32_t prefetch;        /* 1 (default, 0): the next block is copied into shared
                                 memory during the merge; 2: also L2-prefetch the
                                 runner-up candidate's block */
@@ -247,6 +248,13 @@ int sqg_search_uniform(const sqg_index *ix, const float *queries, int nq, int k,
  * how many warps run at once and so how much room the spilled visited sets
  * take; 0 on invalid arguments.  Host call, no device work. */
 size_t sqg_workspace_size_ex(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_search_params *params);
+
+/* What a search with these arguments launches, for tests (host call, no device
+ * work): out[0] = the kernel (0 general, 1 compact, 2 deep-beam), out[1] = log2
+ * of the visited set's shared-memory slots, out[2] = warps per block, out[3] =
+ * the most warps that can be resident per SM. */
+int sqg_search_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_search_params *params,
+                    int32_t out[4]);
 
 /* Query preparation alone (the first kernels of sqg_search), for tests:
  *   out_qrot   nq x d fp32: q' = P^-1 q (Eq. (4)) in the canonical order:

@@ -59,6 +59,7 @@ _SIGS = {
     "sqg_index_info": (I32, [P, C.POINTER(Info)]),
     "sqg_workspace_size": (SZ, [P, I32, I32, I32]),
     "sqg_workspace_size_ex": (SZ, [P, I32, I32, I32, P]),
+    "sqg_search_plan": (I32, [P, I32, I32, I32, C.POINTER(SearchParams), P]),
     "sqg_search": (I32, [P, P, I32, P, P, P, P, P]),
     "sqg_search_ex": (I32, [P, P, I32, P, P, P, P, C.POINTER(SearchParams), P, SZ, P, P]),
     "sqg_search_uniform": (I32, [P, P, I32, I32, I32, P, P, C.POINTER(SearchParams), P, SZ, P, P]),

@@ -408,6 +408,7 @@ int pick_ch(uint32_t d) {
 
 struct LaunchPlan {
     int ch, nb, team, warps, grid;
+    int resident;  // warps per SM
     bool compact;  // the compact kernel (search_compact.cu)
     bool deep;     // the deep-beam kernel (search_deep.cu)
     int lean;      // the compact kernel's build (params.lean, or kLeanIdle)
@@ -507,10 +508,17 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
     // visited set: 2^9 slots in shared memory (more cost resident warps: 2^10
     // is 9 % slower for 16,384 candidate searches at ef 400); a search past
     // half of them moves to its warp's full-size table in the workspace.  A
-    // batch whose queries are all resident at once has no use for more warps:
-    // it takes up to 2^11 slots, which spares it the move and the global probes
-    // (719 queries of d 96: ef 160 492 -> 463 us, ef 400 1,074 -> 1,016; 500 of
-    // d 1536 at ef 400 1,567 -> 1,536).
+    // batch whose queries are all resident at once takes a larger table, which
+    // spares it the move and the global probes, as far as that leaves room for
+    // the batches that other streams run beside it: 2^10 slots where at least
+    // 3/4 of the warps stay resident (d > 256: all of them), 2^11 where no more
+    // go.  us per step, one stream / 8 streams, 2^9 | 2^10 | 2^11 slots:
+    //   719 queries of d 96, ef 160, k 10 and 100 (22 / 18 / 14 warps per SM):
+    //     492 / 103 | 465 / 106 | 464 / 120
+    //   700 of d 128, ef 400 (26 / 20 / 15): 603 / 107 | 588 / 112 | 591 / 132
+    //   500 of d 128, ef 120 (20 / 20 / 18): 201 / 35.1 | 187 / 30.8 | 199 / 34.7
+    //   500 of d 960, ef 112 (12 / 11 / 9): 420 / 145 | 423 / 159 | 417 / 166
+    //   500 of d 1536, ef 200 (12 / 10 / 9): 998 / 235 | 1,048 / 265 | 981 / 271
     a.o_hash = (uint32_t)o;
     const size_t cta = 0;  // the stop network's weights are read from the workspace (L1-cached)
     size_t warp_bytes = 0;
@@ -565,15 +573,19 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
         }
         return SQG_OK;
     };
-    bool sized = false;
-    if (p.visited_smem_log2 == 0 && (pl.compact || pl.deep) && generous && bits > 9)
-        for (uint32_t b : {11u, 10u}) {
-            if (sized || (b == 11u && bits < 11u)) continue;
-            if (residency(b) != SQG_OK) return SQG_ERR_CUDA;
-            sized = (long long)per_sm * warps * ix->num_sms >= nq;
+    if (residency(p.visited_smem_log2 > 0 ? (uint32_t)p.visited_smem_log2 : 9u) != SQG_OK) return SQG_ERR_CUDA;
+    if (p.visited_smem_log2 == 0 && (pl.compact || pl.deep) && generous) {
+        int least = small_d ? (3 * per_sm * warps + 3) / 4 : per_sm * warps;
+        for (uint32_t slots = 10; slots <= std::min<uint32_t>(bits, 11u); ++slots) {
+            if (residency(slots) != SQG_OK) return SQG_ERR_CUDA;
+            const int now = per_sm * warps;
+            if (now < least || (long long)now * ix->num_sms < nq) {  // back to the one before
+                if (residency(slots - 1) != SQG_OK) return SQG_ERR_CUDA;
+                break;
+            }
+            least = now;
         }
-    if (!sized && residency(p.visited_smem_log2 > 0 ? (uint32_t)p.visited_smem_log2 : 9u) != SQG_OK)
-        return SQG_ERR_CUDA;
+    }
     pl.ghash = a.shash_bits < bits;
     if (warps < 1 || per_sm < 1) return SQG_ERR_CAPACITY;
     a.warp_bytes = (uint32_t)warp_bytes;
@@ -581,6 +593,7 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
     pl.warps = warps;
     pl.smem = cta + warps * V * warp_bytes;
     const long long want = ((long long)nq + warps * V - 1) / (warps * V);
+    pl.resident = per_sm * warps;
     pl.grid = (int)std::max(1LL, std::min<long long>((long long)per_sm * ix->num_sms, want));
     // workspace
     size_t w = 0;
@@ -878,6 +891,24 @@ extern "C" size_t sqg_workspace_size_ex(const sqg_index *ix, int nq, int max_k, 
     LaunchPlan pl;
     if (make_plan(ix, nq, max_k, max_ef, p, pl) != SQG_OK) return 0;
     return pl.ws_total;
+}
+
+extern "C" int sqg_search_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_search_params *params,
+                               int32_t out[4]) {
+    if (!ix || !out || nq < 1 || max_k < 1 || max_k > SQG_MAX_K || max_ef < max_k || max_ef > SQG_MAX_EF)
+        return SQG_ERR_INVALID_ARG;
+    sqg_search_params p = params ? *params : default_params();
+    if (params && p.stop_every == 0) p.stop_every = 1;
+    if (check_params(p) != SQG_OK) return SQG_ERR_INVALID_ARG;
+    DeviceGuard g(ix->device);
+    LaunchPlan pl;
+    const int rc = make_plan(ix, nq, max_k, max_ef, p, pl);
+    if (rc != SQG_OK) return rc;
+    out[0] = pl.compact ? 1 : pl.deep ? 2 : 0;
+    out[1] = (int32_t)pl.a.shash_bits;
+    out[2] = pl.warps;
+    out[3] = pl.resident;
+    return SQG_OK;
 }
 
 static int search_impl(const sqg_index *ix, const float *queries, int nq, const int32_t *k, const int32_t *ef,
