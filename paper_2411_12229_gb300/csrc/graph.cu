@@ -407,9 +407,9 @@ __global__ void flood_kernel(const uint32_t *__restrict__ adj, uint64_t n, uint3
 // finished rows go to adj (n x R).
 __global__ void __launch_bounds__(kWarps * 32) adjust_refine_kernel(
     const float *__restrict__ data, uint64_t n, uint32_t d, uint32_t L, uint32_t Rr, const u64 *__restrict__ c_own,
-    const uint32_t *__restrict__ c_cnt, const u64 *__restrict__ k1, const uint32_t *__restrict__ n1,
-    const u64 *__restrict__ rev, const uint64_t *__restrict__ roff, int regular, uint32_t R, u64 *k2, uint32_t *n2,
-    uint32_t *flag, uint32_t *adj, u64 *counters) {
+    const uint32_t *__restrict__ c_cnt, u64 *k1, const uint32_t *__restrict__ n1, const u64 *__restrict__ rev,
+    const uint64_t *__restrict__ roff, int regular, uint32_t R, uint32_t *n2, uint32_t *flag, uint32_t *adj,
+    u64 *counters) {
     __shared__ WarpLists lists[kWarps];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     WarpLists &S = lists[w];
@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(kWarps * 32) adjust_refine_kernel(
         const bool fill = regular && nk < (int)Rr;  // the host adds random vertices
         for (uint32_t t = lane; t < R && !fill; t += 32)
             adj[u * R + t] = t < (uint32_t)nk ? key_id(S.k[t]) : regular ? key_id(S.k[t % nk]) : kNone;
-        for (int i = lane; i < nk && fill; i += 32) k2[u * Rr + i] = S.k[i];
+        for (int i = lane; i < nk && fill; i += 32) k1[u * Rr + i] = S.k[i];  // (its kept edges are in the pool)
         if (lane == 0) {
             n2[u] = (uint32_t)nk;
             flag[u] = fill ? kFlagFill : 0u;
@@ -552,18 +552,17 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
     }
     int rc = SQG_OK;
     {
-        // What is not needed at the same time shares memory: the rows, and the
-        // reverse lists where they fit behind them, take the candidate ids'
-        // place once the pruning has read those; the reverse counts, the kept
-        // edges' counts and the flood's levels follow one another.  The reverse
-        // lists are allocated at their real length, about a third of n R'.
-        DevArena A, V;
+        // What is not needed at the same time shares memory: the rows take the
+        // candidate ids' place once the pruning has read those, a row left to the
+        // host its kept edges'; the reverse counts, the refined lists' counts and
+        // the flood's levels follow one another.
+        DevArena A;
         const size_t cand_bytes = sizeof(uint32_t) * n * L;
         const size_t rows_bytes = (sizeof(uint32_t) * n * R + 255) / 256 * 256;
         const size_t o_data = A.add(sizeof(float) * n * d), o_cand = A.add(std::max(cand_bytes, rows_bytes));
         const size_t o_own = A.add(sizeof(u64) * n * L), o_cnt = A.add(sizeof(uint32_t) * n);
         const size_t o_k1 = A.add(sizeof(u64) * n * Rr), o_n1 = A.add(sizeof(uint32_t) * n);
-        const size_t o_roff = A.add(sizeof(uint64_t) * (n + 1)), o_k2 = A.add(sizeof(u64) * n * Rr);
+        const size_t o_roff = A.add(sizeof(uint64_t) * (n + 1)), o_rev = A.add(sizeof(u64) * n * Rr);
         const size_t o_n2 = A.add(sizeof(uint32_t) * n), o_flag = A.add(sizeof(uint32_t) * n);
         constexpr int kBatch = 8;  // flood levels between looks at the result
         const size_t o_ctr = A.add(sizeof(u64) * kCounters), o_grew = A.add(sizeof(uint32_t) * kBatch);
@@ -575,7 +574,7 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
         uint32_t *c_cnt = A.at<uint32_t>(o_cnt), *n1 = A.at<uint32_t>(o_n1), *flag = A.at<uint32_t>(o_flag);
         uint32_t *d_cand = A.at<uint32_t>(o_cand), *d_adj = d_cand;
         uint32_t *n2 = A.at<uint32_t>(o_n2), *rcnt = n2, *level = n2;
-        u64 *c_own = A.at<u64>(o_own), *k1 = A.at<u64>(o_k1), *k2 = A.at<u64>(o_k2), *d_rev = nullptr;
+        u64 *c_own = A.at<u64>(o_own), *k1 = A.at<u64>(o_k1), *d_rev = A.at<u64>(o_rev);
         uint64_t *d_roff = A.at<uint64_t>(o_roff);
         u64 *ctr = A.at<u64>(o_ctr), h_ctr[kCounters] = {};
         int sms = 0;
@@ -596,28 +595,12 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
             ok(cudaMemcpy(h_ctr, ctr, sizeof(h_ctr), cudaMemcpyDeviceToHost));
             if (rc == SQG_OK && h_ctr[kBadValues]) rc = SQG_ERR_INVALID_ARG;
         }
-        if (rc == SQG_OK) {  // (1), and the reverse lists' lengths
+        if (rc == SQG_OK) {  // (1)-(3)
             adjust_prune_kernel<<<grid, kWarps * 32>>>(d_data, n, d, d_cand, L, Rr, c_own, c_cnt, k1, n1, rcnt, ctr);
             reverse_offsets_kernel<<<1, kScanThreads>>>(rcnt, n, d_roff);
-            ok(cudaGetLastError());
-            ok(cudaMemcpy(h_ctr, ctr, sizeof(h_ctr), cudaMemcpyDeviceToHost));  // (the pruning is done)
-            const size_t rev_bytes = sizeof(u64) * h_ctr[kSumKept];
-            if (rows_bytes + rev_bytes <= cand_bytes) {
-                d_rev = A.at<u64>(o_cand + rows_bytes);
-            } else {
-                V.add(rev_bytes);
-                if (V.commit()) {
-                    d_rev = V.at<u64>(0);
-                } else {
-                    cudaGetLastError();
-                    if (rc == SQG_OK) rc = SQG_ERR_OOM;
-                }
-            }
-        }
-        if (rc == SQG_OK) {  // (2)-(3)
             reverse_fill_kernel<<<warp_blocks, 256>>>(k1, n1, n, Rr, d_roff, rcnt, d_rev);
             adjust_refine_kernel<<<grid, kWarps * 32>>>(d_data, n, d, L, Rr, c_own, c_cnt, k1, n1, d_rev, d_roff,
-                                                        regular ? 1 : 0, R, k2, n2, flag, d_adj, ctr);
+                                                        regular ? 1 : 0, R, n2, flag, d_adj, ctr);
             ok(cudaGetLastError());
             ok(cudaMemcpy(out_adj, d_adj, sizeof(uint32_t) * n * R, cudaMemcpyDeviceToHost));
             ok(cudaMemcpy(h_ctr, ctr, sizeof(h_ctr), cudaMemcpyDeviceToHost));
@@ -626,23 +609,18 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
         const bool host_rows = h_ctr[kHostRows] != 0, fill_rows = h_ctr[kFillRows] != 0;
         if (rc == SQG_OK && (host_rows || fill_rows)) {  // the rows that the kernels left: refine, random fill
             std::vector<uint32_t> h_flag(n), h_n1(n), h_n2(n);
-            std::vector<u64> h_k1, h_rev, h_k2;
+            std::vector<u64> h_k1((size_t)n * Rr), h_rev;  // kept edges of the rows to refine, refined lists of the others
             std::vector<uint64_t> roff;
             ok(cudaMemcpy(h_flag.data(), flag, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost));
+            ok(cudaMemcpy(h_k1.data(), k1, sizeof(u64) * h_k1.size(), cudaMemcpyDeviceToHost));
             if (host_rows) {
-                h_k1.resize((size_t)n * Rr);
                 h_rev.resize((size_t)h_ctr[kSumKept]);
                 roff.resize(n + 1);
-                ok(cudaMemcpy(h_k1.data(), k1, sizeof(u64) * h_k1.size(), cudaMemcpyDeviceToHost));
                 ok(cudaMemcpy(h_n1.data(), n1, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost));
                 ok(cudaMemcpy(roff.data(), d_roff, sizeof(uint64_t) * (n + 1), cudaMemcpyDeviceToHost));
                 ok(cudaMemcpy(h_rev.data(), d_rev, sizeof(u64) * h_rev.size(), cudaMemcpyDeviceToHost));
             }
-            if (fill_rows) {
-                h_k2.resize((size_t)n * Rr);
-                ok(cudaMemcpy(h_k2.data(), k2, sizeof(u64) * h_k2.size(), cudaMemcpyDeviceToHost));
-                ok(cudaMemcpy(h_n2.data(), n2, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost));
-            }
+            if (fill_rows) ok(cudaMemcpy(h_n2.data(), n2, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost));
             std::vector<uint64_t> left;
             for (uint64_t u = 0; u < n; ++u)
                 if (h_flag[u]) left.push_back(u);
@@ -658,7 +636,7 @@ extern "C" int sqg_build_graph_ex(const float *data, uint64_t n, uint32_t d, con
                                                      rev.size(), regular, l2))
                             n_supp++;
                     } else {
-                        for (uint32_t j = 0; j < h_n2[u]; ++j) l2.push_back(unpack_host(h_k2[u * Rr + j]));
+                        for (uint32_t j = 0; j < h_n2[u]; ++j) l2.push_back(unpack_host(h_k1[u * Rr + j]));
                     }
                     if (sqg_graph::fill_and_write(data, n, d, R, Rr, seed, u, regular, l2, out_adj)) n_fill++;
                 }, 1);
