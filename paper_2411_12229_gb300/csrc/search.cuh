@@ -236,20 +236,29 @@ struct QuerySide {
     int sq;
 };
 // Team T: coordinate 32w + tl + T v belongs to lane tl (v < 32/T); the
-// planes' word w is assembled from the 32/T team ballots.
-template <int T>
+// planes' word w is assembled from the 32/T team ballots.  ONE: one word at a
+// time, a chain of d / 32 loads, for the kernels for d <= 256, whose registers
+// it keeps (96 against 110 in the build for few queries); longer rows take 1.5
+// to 3 times as long that way (1,000 queries: d 480 4.4 -> 8.1 us, d 1024 4.5 ->
+// 9.6, d 1536 6.7 -> 22.3).
+template <int T, bool ONE = false>
 __device__ __forceinline__ QuerySide quantize_team(const float *qr, uint32_t d, uint32_t *planes, const Team<T> &tm) {
     constexpr int V = Team<T>::V;
     const uint32_t nw = d / 32;
     float vl = __int_as_float(0x7f800000), vr = -vl;
-#pragma unroll 1
-    for (uint32_t w = 0; w < nw; ++w) {
+    auto extremes = [&](uint32_t w) {
 #pragma unroll
         for (int v = 0; v < V; ++v) {
             const float x = qr[w * 32 + tm.tl + T * v];
             vl = x < vl ? x : vl;
             vr = x > vr ? x : vr;
         }
+    };
+    if constexpr (ONE) {
+#pragma unroll 1
+        for (uint32_t w = 0; w < nw; ++w) extremes(w);
+    } else {
+        for (uint32_t w = 0; w < nw; ++w) extremes(w);
     }
 #pragma unroll
     for (int o = T / 2; o >= 1; o >>= 1) {
@@ -264,8 +273,7 @@ __device__ __forceinline__ QuerySide quantize_team(const float *qr, uint32_t d, 
     const float inv = range > 0.0f ? __fdiv_rn(15.0f, range) : 0.0f;
     qs.inv_sqrt_d = __fdiv_rn(1.0f, __fsqrt_rn((float)d));
     int sq = 0;
-#pragma unroll 1
-    for (uint32_t w = 0; w < nw; ++w) {
+    auto word = [&](uint32_t w) {
         uint32_t b0 = 0, b1 = 0, b2 = 0, b3 = 0;
 #pragma unroll
         for (int v = 0; v < V; ++v) {
@@ -287,6 +295,12 @@ __device__ __forceinline__ QuerySide quantize_team(const float *qr, uint32_t d, 
             // word-major: the 4 planes of word w share one 16-byte slot
             reinterpret_cast<uint4 *>(planes)[w] = make_uint4(b0, b1, b2, b3);
         }
+    };
+    if constexpr (ONE) {
+#pragma unroll 1
+        for (uint32_t w = 0; w < nw; ++w) word(w);
+    } else {
+        for (uint32_t w = 0; w < nw; ++w) word(w);
     }
     qs.sq = tm.reduce_add(sq);
     return qs;

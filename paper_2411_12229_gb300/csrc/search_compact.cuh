@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(128, MINB) search_compact_kernel(const SearchA
             qs.sq = (int)sc.z;
             qs.inv_sqrt_d = sc.w;
         } else {
-            qs = quantize_team<32>(a.qrot + (size_t)qi * d, d, planes, tm);
+            qs = quantize_team<32, CH <= 2>(a.qrot + (size_t)qi * d, d, planes, tm);
         }
         uint32_t *H = Hs;
         uint32_t hbits = a.shash_bits;
