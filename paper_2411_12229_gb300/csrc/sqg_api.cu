@@ -509,16 +509,17 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
     // is 9 % slower for 16,384 candidate searches at ef 400); a search past
     // half of them moves to its warp's full-size table in the workspace.  A
     // batch whose queries are all resident at once takes a larger table, which
-    // spares it the move and the global probes, as far as that leaves room for
-    // the batches that other streams run beside it: 2^10 slots where at least
-    // 3/4 of the warps stay resident (d > 256: all of them), 2^11 where no more
-    // go.  us per step, one stream / 8 streams, 2^9 | 2^10 | 2^11 slots:
-    //   719 queries of d 96, ef 160, k 10 and 100 (22 / 18 / 14 warps per SM):
+    // spares it the move and the global probes; the warps it gives up are missed
+    // by batches that other streams run beside it.  So in the compact kernel 2^10
+    // slots are taken where at least 3/4 of the warps stay (d > 256: all of them)
+    // and 2^11 where no more go; in the deep kernel up to 2^11.  us per batch, one
+    // stream / 8 streams, with 2^9 | 2^10 | 2^11 slots (warps per SM):
+    //   719 queries of d 96, ef 160, k 10 and 100 (22 / 18 / 14):
     //     492 / 103 | 465 / 106 | 464 / 120
-    //   700 of d 128, ef 400 (26 / 20 / 15): 603 / 107 | 588 / 112 | 591 / 132
     //   500 of d 128, ef 120 (20 / 20 / 18): 201 / 35.1 | 187 / 30.8 | 199 / 34.7
     //   500 of d 960, ef 112 (12 / 11 / 9): 420 / 145 | 423 / 159 | 417 / 166
-    //   500 of d 1536, ef 200 (12 / 10 / 9): 998 / 235 | 1,048 / 265 | 981 / 271
+    //   deep, 700 of d 128, ef 400 (26 / 20 / 15): 603 / 107 | 588 / 112 | 580 / 133
+    //   deep, 500 of d 1536, ef 200 (12 / 10 / 9): 998 / 235 | 1,048 / 265 | 971 / 261
     a.o_hash = (uint32_t)o;
     const size_t cta = 0;  // the stop network's weights are read from the workspace (L1-cached)
     size_t warp_bytes = 0;
@@ -575,7 +576,7 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
     };
     if (residency(p.visited_smem_log2 > 0 ? (uint32_t)p.visited_smem_log2 : 9u) != SQG_OK) return SQG_ERR_CUDA;
     if (p.visited_smem_log2 == 0 && (pl.compact || pl.deep) && generous) {
-        int least = small_d ? (3 * per_sm * warps + 3) / 4 : per_sm * warps;
+        int least = pl.deep ? 0 : small_d ? (3 * per_sm * warps + 3) / 4 : per_sm * warps;
         for (uint32_t slots = 10; slots <= std::min<uint32_t>(bits, 11u); ++slots) {
             if (residency(slots) != SQG_OK) return SQG_ERR_CUDA;
             const int now = per_sm * warps;
@@ -583,7 +584,7 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
                 if (residency(slots - 1) != SQG_OK) return SQG_ERR_CUDA;
                 break;
             }
-            least = now;
+            if (pl.compact) least = now;
         }
     }
     pl.ghash = a.shash_bits < bits;

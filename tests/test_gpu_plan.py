@@ -64,7 +64,7 @@ def test_larger_tables_leave_room(tmp_path, lib_built, d, R):
     larger = 0
     for k, ef in ((1, 1), (10, 40), (10, 64), (10, 120), (10, 200), (100, 160), (100, 256), (10, 400), (128, 1000)):
         for nq in (1, 200, 719, 8 * sms, 8 * sms + 1, 2001, 3000, 10_000):
-            kernel, slots, _, resident = plan(nq, k, ef)
+            kernel, slots, _, resident = plan(nq, k, ef)  # (the deep kernel's rule is residency alone)
             least = plan(nq, k, ef, 9)
             assert kernel in (1, 2) and slots <= 11 and least[1] <= 9
             if slots <= 9:
@@ -72,6 +72,7 @@ def test_larger_tables_leave_room(tmp_path, lib_built, d, R):
                 continue
             larger += 1
             assert nq <= resident * sms
-            assert 4 * resident >= 3 * least[3] if d <= 256 else resident == least[3]
-            assert slots == 10 or resident == plan(nq, k, ef, 10)[3]
+            if kernel == 1:
+                assert 4 * resident >= 3 * least[3] if d <= 256 else resident == least[3]
+                assert slots == 10 or resident == plan(nq, k, ef, 10)[3]
     assert larger > 0
