@@ -22,8 +22,8 @@
 // reduce-scatter that leaves one pair per lane (31 shuffles for 32 pairs
 // instead of 160), and each lane then takes its own pair's cosine.
 // Measured at 20,000 vertices of d 128, R = 32, 96 candidates: refinement
-// 18.4 -> 3.1 ms, pruning 1.80 -> 1.25 ms; the whole call 28.2 -> 5.3 ms with
-// the reverse lists (host loops over all edges before), the rows and the
+// 18.4 -> 3.1 ms, pruning 1.80 -> 1.23 ms; the whole call 28-30 -> 4.9-5.4 ms
+// with the reverse lists (host loops over all edges before), the rows and the
 // flood on the device as well.
 #include <cuda_runtime.h>
 

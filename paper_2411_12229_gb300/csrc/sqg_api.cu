@@ -454,7 +454,9 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
     pl.crk = max_k <= 32 ? 1 : 4;
     // Up to eight queries per SM leave most issue slots free: a build with twice
     // the registers and shorter chains (one query of d 128: 73 -> 65 us, 200: 92
-    // -> 79, 1,200: 133 -> 114, at ef 100 186 -> 170).
+    // -> 79, 1,200: 133 -> 114, at ef 100 186 -> 170).  Batches side by side on
+    // several streams take about the same with either build (16 streams of 200
+    // queries 10.0 -> 9.8 us per batch, 8 of 1,000 29.8 -> 30.9).
     pl.lean = p.lean == 0 && pl.ch <= 2 && pl.nb == 1 && nq <= 8 * ix->num_sms ? kLeanIdle : p.lean;
     const bool big = pl.compact && (pl.cbnb == 8 || pl.crk == 4);  // search_compact_big.cu
     if (pl.compact || pl.deep) {
