@@ -97,10 +97,11 @@ typedef struct {
     void *timing_events[2];  /* optional cudaEvent_t pair recorded on the stream right before
                                 and right after the search kernel; NULL = none */
     int32_t visited_smem_log2; /* log2 of the visited set's shared-memory slots (5..12;
-                                  0 = 9, or 10 or 11 for a batch whose queries are all
-                                  resident at once, in the compact kernel as far as few or
-                                  no resident warps are given up for it); a search past half
-                                  of them continues in a full-size table in the workspace */
+                                  0 = 9, or 10 or 11 for a batch without the stop whose
+                                  queries are all resident at once, in the compact kernel as
+                                  far as few or no resident warps are given up for it); a
+                                  search past half of them continues in a full-size table in
+                                  the workspace */
     int32_t prefetch;        /* 1 (default, 0): the next block is copied into shared
                                 memory during the merge; 2: also L2-prefetch the
                                 runner-up candidate's block */

@@ -514,7 +514,9 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
     // spares it the move and the global probes; the warps it gives up are missed
     // by batches that other streams run beside it.  So in the compact kernel 2^10
     // slots are taken where at least 3/4 of the warps stay (d > 256: all of them)
-    // and 2^11 where no more go; in the deep kernel up to 2^11.  us per batch, one
+    // and 2^11 where no more go; in the deep kernel up to 2^11; none with the stop,
+    // whose network is read through the L1 that the tables take (700 queries of d
+    // 128, ef 96, one stream / 8: 2^9 273 / 56.9, 2^10 289 / 59.2).  us per batch, one
     // stream / 8 streams, with 2^9 | 2^10 | 2^11 slots (warps per SM):
     //   719 queries of d 96, ef 160, k 10 and 100 (22 / 18 / 14):
     //     492 / 103 | 465 / 106 | 464 / 120
@@ -577,7 +579,7 @@ int make_plan(const sqg_index *ix, int nq, int max_k, int max_ef, const sqg_sear
         return SQG_OK;
     };
     if (residency(p.visited_smem_log2 > 0 ? (uint32_t)p.visited_smem_log2 : 9u) != SQG_OK) return SQG_ERR_CUDA;
-    if (p.visited_smem_log2 == 0 && (pl.compact || pl.deep) && generous) {
+    if (p.visited_smem_log2 == 0 && (pl.compact || pl.deep) && generous && !p.stop_mlp) {
         int least = pl.deep ? 0 : small_d ? (3 * per_sm * warps + 3) / 4 : per_sm * warps;
         for (uint32_t slots = 10; slots <= std::min<uint32_t>(bits, 11u); ++slots) {
             if (residency(slots) != SQG_OK) return SQG_ERR_CUDA;

@@ -55,18 +55,20 @@ def test_larger_tables_leave_room(tmp_path, lib_built, d, R):
     ix = Index(p, 0)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
 
-    def plan(nq, k, ef, slots=0):
+    def plan(nq, k, ef, slots=0, **kw):
         out = (C.c_int32 * 4)()
-        params = ix.params(visited_smem_log2=slots)
+        params = ix.params(visited_smem_log2=slots, **kw)
         B.check(B.lib().sqg_search_plan(ix.handle, nq, k, ef, C.byref(params), out), "sqg_search_plan")
         return list(out)
 
+    stop = torch.zeros(B.MLP_NPARAM, device="cuda")
     larger = 0
     for k, ef in ((1, 1), (10, 40), (10, 64), (10, 120), (10, 200), (100, 160), (100, 256), (10, 400), (128, 1000)):
         for nq in (1, 200, 719, 8 * sms, 8 * sms + 1, 2001, 3000, 10_000):
             kernel, slots, _, resident = plan(nq, k, ef)  # (the deep kernel's rule is residency alone)
             least = plan(nq, k, ef, 9)
             assert kernel in (1, 2) and slots <= 11 and least[1] <= 9
+            assert plan(nq, k, ef, stop_mlp=stop)[1] <= 9
             if slots <= 9:
                 assert resident == least[3]
                 continue
