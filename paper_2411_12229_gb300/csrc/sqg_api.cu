@@ -197,22 +197,22 @@ __global__ void mlp_transpose_kernel(const float *__restrict__ src, float *__res
 // RPT - 1, lane l outputs l + 32 j; every output walks j in order with one
 // chunk accumulator and one total, so the tiling changes no bit.
 //
-// Slabs of up to 128 columns of the tile's queries and rows of P^-1 are staged
-// as they are (16-byte copies, rows padded to 132 floats); a step of four j
+// Slabs of up to SLAB columns of the tile's queries and rows of P^-1 are staged
+// as they are (16-byte copies, rows padded by 4 floats); a step of four j
 // reads one float4 per query (a broadcast) and per output (a bank quad each).
 // With RPT = 8, CPT = 4 that is 12 reads for 128 multiply-adds.  us at d 128
 // for 1 / 200 / 2,001 / 10,000 / 50,000 queries: 2.9 / 3.1 / 5.1 / 15.1 / 48.1;
 // 6.8 / 7.4 / 7.5 / 17.7 / 59.2 with one 64 x 64 tile size staged transposed.
 // A copy group per chunk, waited for one by one, was 2-10 % slower.
-constexpr int kRotSlab = 128, kRotPitch = kRotSlab + 4, kRotWarps = 8;
-template <int RPT, int CPT>
+constexpr int kRotWarps = 8;
+template <int RPT, int CPT, int SLAB>
 __global__ void __launch_bounds__(kRotWarps * 32) rotate_kernel(const float *__restrict__ q,
                                                                 const float *__restrict__ rot,
                                                                 float *__restrict__ out, int nq, int d,
                                                                 unsigned int *queue) {
-    constexpr int kRows = kRotWarps * RPT, kCols = 32 * CPT;
+    constexpr int kRows = kRotWarps * RPT, kCols = 32 * CPT, kPitch = SLAB + 4;
     extern __shared__ __align__(16) float rot_smem[];
-    float *const qs = rot_smem, *const ps = rot_smem + kRows * kRotPitch;
+    float *const qs = rot_smem, *const ps = rot_smem + kRows * kPitch;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int r0 = blockIdx.y * kRows, c0 = blockIdx.x * kCols;
     if (queue && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *queue = 0u;  // the search's work queue
@@ -221,18 +221,18 @@ __global__ void __launch_bounds__(kRotWarps * 32) rotate_kernel(const float *__r
     for (int i = 0; i < RPT; ++i)
 #pragma unroll
         for (int j = 0; j < CPT; ++j) tot[i][j] = 0.0f;
-    for (int k0 = 0; k0 < d; k0 += kRotSlab) {
-        const int width = min(kRotSlab, d - k0);  // a multiple of 32
-        if (k0 > 0) __syncthreads();              // the last slab's reads
+    for (int k0 = 0; k0 < d; k0 += SLAB) {
+        const int width = min(SLAB, d - k0);  // a multiple of 32
+        if (k0 > 0) __syncthreads();         // the last slab's reads
         // (rows past the ends are left as they are: their outputs are not written)
-        for (int e = tid; e < (kRows + kCols) * (kRotSlab / 4); e += kRotWarps * 32) {
-            const int row = e / (kRotSlab / 4), col = 4 * (e % (kRotSlab / 4));
+        for (int e = tid; e < (kRows + kCols) * (SLAB / 4); e += kRotWarps * 32) {
+            const int row = e / (SLAB / 4), col = 4 * (e % (SLAB / 4));
             const bool is_q = row < kRows;
             const int gr = is_q ? r0 + row : c0 + row - kRows;
             if (col < width && gr < (is_q ? nq : d)) {
                 const float *src = (is_q ? q : rot) + (size_t)gr * d + k0 + col;
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                                 smem_addr(rot_smem + row * kRotPitch + col)),
+                                 smem_addr(rot_smem + row * kPitch + col)),
                              "l"(src)
                              : "memory");
             }
@@ -250,10 +250,10 @@ __global__ void __launch_bounds__(kRotWarps * 32) rotate_kernel(const float *__r
                 float4 pv[CPT];
 #pragma unroll
                 for (int j = 0; j < CPT; ++j)
-                    pv[j] = *reinterpret_cast<const float4 *>(ps + (lane + 32 * j) * kRotPitch + k);
+                    pv[j] = *reinterpret_cast<const float4 *>(ps + (lane + 32 * j) * kPitch + k);
 #pragma unroll
                 for (int i = 0; i < RPT; ++i) {
-                    const float4 v = *reinterpret_cast<const float4 *>(qs + (w * RPT + i) * kRotPitch + k);
+                    const float4 v = *reinterpret_cast<const float4 *>(qs + (w * RPT + i) * kPitch + k);
 #pragma unroll
                     for (int j = 0; j < CPT; ++j) {
                         acc[i][j] = __fmaf_rn(pv[j].x, v.x, acc[i][j]);
@@ -281,12 +281,12 @@ __global__ void __launch_bounds__(kRotWarps * 32) rotate_kernel(const float *__r
     }
 }
 
-template <int RPT, int CPT>
+template <int RPT, int CPT, int SLAB>
 cudaError_t launch_rotate(const float *q, const float *rot, float *out, int nq, int d, unsigned int *queue,
                           cudaStream_t s) {
     constexpr int kRows = kRotWarps * RPT, kCols = 32 * CPT;
-    constexpr int smem = (kRows + kCols) * kRotPitch * (int)sizeof(float);
-    auto fn = rotate_kernel<RPT, CPT>;
+    constexpr int smem = (kRows + kCols) * (SLAB + 4) * (int)sizeof(float);
+    auto fn = rotate_kernel<RPT, CPT, SLAB>;
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     fn<<<dim3((d + kCols - 1) / kCols, (nq + kRows - 1) / kRows), kRotWarps * 32, smem, s>>>(q, rot, out, nq, d, queue);
@@ -645,11 +645,20 @@ cudaError_t rotate_simt(const sqg_index *ix, const float *queries, float *out, i
     // tiles; 20,000: 25.3 against 24.6).  Up to two 8 x 32 tiles per SM the
     // launch is one tile's chain of d multiply-adds and the small tile's load is
     // the shortest (200 queries: 3.1 against 4.6; 719, past the line: 5.0
-    // against 4.7).
+    // against 4.7).  Below four 32 x 64 tiles per SM the slabs are of 64 columns:
+    // 26 KB of shared memory instead of 51 find room sooner beside the search
+    // blocks of other streams' batches (3 streams of 5,000 queries, ef 64 133 ->
+    // 131 us per batch, with the stop at ef 96 304 -> 292; 4 of 1,216 43.1 ->
+    // 40.5; alone 10.0 -> 10.8 us for 5,000).  Larger launches gain nothing by it
+    // (3 of 10,000: 189.5 against 190.8).
     auto blocks = [&](long long rows, long long cols) { return ((nq + rows - 1) / rows) * ((d + cols - 1) / cols); };
-    if (blocks(64, 128) >= 4LL * ix->num_sms) return launch_rotate<8, 4>(queries, ix->d_rot, out, nq, d, queue, stream);
-    if (blocks(8, 32) > 2LL * ix->num_sms) return launch_rotate<4, 2>(queries, ix->d_rot, out, nq, d, queue, stream);
-    return launch_rotate<1, 1>(queries, ix->d_rot, out, nq, d, queue, stream);
+    if (blocks(64, 128) >= 4LL * ix->num_sms)
+        return launch_rotate<8, 4, 128>(queries, ix->d_rot, out, nq, d, queue, stream);
+    if (blocks(32, 64) >= 4LL * ix->num_sms)
+        return launch_rotate<4, 2, 128>(queries, ix->d_rot, out, nq, d, queue, stream);
+    if (blocks(8, 32) > 2LL * ix->num_sms)
+        return launch_rotate<4, 2, 64>(queries, ix->d_rot, out, nq, d, queue, stream);
+    return launch_rotate<1, 1, 128>(queries, ix->d_rot, out, nq, d, queue, stream);
 }
 
 // Rotation path: 1 = the CUDA-core kernel in the canonical order, 2 = tensor

@@ -1,6 +1,7 @@
 """The dispatch lines that follow the GPU's number of SMs, on the SMs of the
 GPU at hand: searches of 8 queries per SM and one more (the build for few
-queries), gradients of one tile per SM and one sample more."""
+queries), rotations on both sides of four 32 x 64 tiles per SM, gradients of
+one tile per SM and one sample more."""
 
 import numpy as np
 import pytest
@@ -28,6 +29,28 @@ def test_searches(tmp_path, lib_built, sms, d):
         for nq in (8 * sms - 1, 8 * sms, 8 * sms + 1):
             got = ix.search(q[:nq], k, ef, stats=True, kernel=2)
             assert all(torch.equal(a, b[:nq]) for a, b in zip(got, ref))
+
+
+@pytest.mark.parametrize("d", [32, 64, 96, 128, 160, 256, 480])
+def test_rotations(tmp_path, lib_built, sms, d):
+    """The staging of a tile changes no bit: batches on both sides of the line
+    against the same rows in calls of eight."""
+    from paper_2411_12229_gb300 import index_builder as ib
+    from paper_2411_12229_gb300 import synth
+    from paper_2411_12229_gb300.api import Index
+    w = synth.small(synth.BATCHED_1M_D128.with_(d=d), 200, 1)
+    p = tmp_path / "i.sqg"
+    ib.build_index(p, synth.base(w), 32)
+    ix = Index(p, 0)
+    line = 32 * -(-4 * sms // -(-d // 64))  # the most queries below the line, and those of the tile before
+    q = torch.randn((line + 64, d), device="cuda", generator=torch.Generator(device="cuda").manual_seed(d))
+    rows = range(0, line + 64, max(8, line // 40 // 8 * 8))
+    ref = {i: ix.prepare_queries(q[i:i + 8].contiguous()) for i in rows}
+    for nq in (line - 32, line - 31, line, line + 33, line + 64):
+        got = ix.prepare_queries(q[:nq].contiguous())
+        for i in rows:
+            if i + 8 <= nq:
+                assert all(torch.equal(a[i:i + 8], b) for a, b in zip(got, ref[i]))
 
 
 @pytest.mark.parametrize("more", [-1, 0, 1])
