@@ -201,7 +201,7 @@ __global__ void mlp_transpose_kernel(const float *__restrict__ src, float *__res
 // as they are (16-byte copies, rows padded by 4 floats); a step of four j
 // reads one float4 per query (a broadcast) and per output (a bank quad each).
 // With RPT = 8, CPT = 4 that is 12 reads for 128 multiply-adds.  us at d 128
-// for 1 / 200 / 2,001 / 10,000 / 50,000 queries: 2.9 / 3.1 / 5.1 / 15.1 / 48.1;
+// for 1 / 200 / 2,001 / 10,000 / 50,000 queries: 2.7 / 3.2 / 5.9 / 15.1 / 48.2;
 // 6.8 / 7.4 / 7.5 / 17.7 / 59.2 with one 64 x 64 tile size staged transposed.
 // A copy group per chunk, waited for one by one, was 2-10 % slower.
 constexpr int kRotWarps = 8;
@@ -645,7 +645,7 @@ cudaError_t rotate_simt(const sqg_index *ix, const float *queries, float *out, i
     // tiles; 20,000: 25.3 against 24.6).  Up to two 8 x 32 tiles per SM the
     // launch is one tile's chain of d multiply-adds and the small tile's load is
     // the shortest (200 queries: 3.1 against 4.6; 719, past the line: 5.0
-    // against 4.7).  Below four 32 x 64 tiles per SM the slabs are of 64 columns:
+    // against 4.7, then with slabs of 128 columns).  Below four 32 x 64 tiles per SM the slabs are of 64 columns:
     // 26 KB of shared memory instead of 51 find room sooner beside the search
     // blocks of other streams' batches (3 streams of 5,000 queries, ef 64 133 ->
     // 131 us per batch, with the stop at ef 96 304 -> 292; 4 of 1,216 43.1 ->
